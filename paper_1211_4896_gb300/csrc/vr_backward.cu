@@ -270,8 +270,9 @@ __global__ void __launch_bounds__(kBwdThreads, BwdMinBlocks<VT>::value) bwd_kern
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 8 + (lane & 7);
-        const int j = (int)(tile / tiles_x) * 4 + (lane >> 3);
+        const int2 at = tile_pixel(lane, 3);
+        const int i = (int)(tile % tiles_x) * 8 + at.x;
+        const int j = (int)(tile / tiles_x) * 4 + at.y;
         Ray ray;
         int n = 0;
         float4 g = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -4,8 +4,8 @@
 // RGBA transfer function and composite front to back, stopping early once the
 // accumulated opacity reaches the threshold.
 //
-// GB300 mapping: persistent warps, one 8x4 pixel tile per warp at a time,
-// pulled from a global atomic queue (load balance across uneven ray lengths
+// GB300 mapping: persistent warps, one 8x4 pixel tile per warp at a time (its
+// lanes in 2x2 quads), pulled from a global atomic queue (load balance across uneven ray lengths
 // and early termination); voxel gathers go through the read-only L1 path from
 // bricks (+apron) so all eight corners of a cell are at constant offsets in
 // one brick, with the next sample's gathers in flight while the current one
@@ -38,18 +38,20 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
                                                            unsigned ntiles)
 {
     const int lane = threadIdx.x & 31;
+    const float z = skips_transparent<T, IdentityMap>() ? transparent_below(p) : 0.0f;
     for (;;) {
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 8 + (lane & 7);
-        const int j = (int)(tile / tiles_x) * 4 + (lane >> 3);
+        const int2 at = tile_pixel(lane, 3);
+        const int i = (int)(tile % tiles_x) * 8 + at.x;
+        const int j = (int)(tile / tiles_x) * 4 + at.y;
         const bool inside = i < c.W && j < c.H;
         Ray ray;
         const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
-        const int used = march_ray<T, LOG2B, L, IdentityMap, FwdDepth<T>::value>(v, p, ray, hit, acc);
+        const int used = march_ray<T, LOG2B, L, IdentityMap, FwdDepth<T>::value>(v, p, ray, hit, acc, z);
         if (inside) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
     }
 }
@@ -68,8 +70,9 @@ __global__ void __launch_bounds__(kFwdThreads) fwd_tex_kernel(cudaTextureObject_
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 8 + (lane & 7);
-        const int j = (int)(tile / tiles_x) * 4 + (lane >> 3);
+        const int2 at = tile_pixel(lane, 3);
+        const int i = (int)(tile % tiles_x) * 8 + at.x;
+        const int j = (int)(tile / tiles_x) * 4 + at.y;
         const bool inside = i < c.W && j < c.H;
         Ray ray;
         const bool hit = inside && setup_ray(c, nx, ny, nz, p.step, i, j, ray);

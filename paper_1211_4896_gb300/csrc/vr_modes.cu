@@ -76,8 +76,9 @@ __global__ void __launch_bounds__(kModeThreads, ModeMinBlocks<T>::value) mip_ker
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 8 + (lane & 7);
-        const int j = (int)(tile / tiles_x) * 4 + (lane >> 3);
+        const int2 at = tile_pixel(lane, 3);
+        const int i = (int)(tile % tiles_x) * 8 + at.x;
+        const int j = (int)(tile / tiles_x) * 4 + at.y;
         const bool inside = i < c.W && j < c.H;
         Ray ray;
         const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
@@ -162,18 +163,20 @@ __global__ void __launch_bounds__(kModeThreads) sigma_kernel(VolDev v, CamDev c,
 {
     const int lane = threadIdx.x & 31;
     const SigmaMap map{m};
+    const float z = skips_transparent<T, SigmaMap>() ? transparent_below(p) : 0.0f;
     for (;;) {
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 8 + (lane & 7);
-        const int j = (int)(tile / tiles_x) * 4 + (lane >> 3);
+        const int2 at = tile_pixel(lane, 3);
+        const int i = (int)(tile % tiles_x) * 8 + at.x;
+        const int j = (int)(tile / tiles_x) * 4 + at.y;
         const bool inside = i < c.W && j < c.H;
         Ray ray;
         const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
-        const int used = march_ray<T, LOG2B, L, SigmaMap>(v, p, ray, hit, acc, map);
+        const int used = march_ray<T, LOG2B, L, SigmaMap>(v, p, ray, hit, acc, z, map);
         if (inside) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
     }
 }
@@ -284,8 +287,9 @@ __global__ void __launch_bounds__(kModeThreads) subbox_kernel(VolDev v, CamDev c
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 8 + (lane & 7);
-        const int j = (int)(tile / tiles_x) * 4 + (lane >> 3);
+        const int2 at = tile_pixel(lane, 3);
+        const int i = (int)(tile % tiles_x) * 8 + at.x;
+        const int j = (int)(tile / tiles_x) * 4 + at.y;
         const bool inside_img = i < c.W && j < c.H;
         Ray ray;
         // rays and samples of the whole grid (gdim voxels; the camera is in its

@@ -153,8 +153,9 @@ __global__ void __launch_bounds__(kSkipThreads) skip_kernel(VolDev v, CamDev c, 
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 8 + (lane & 7);
-        const int j = (int)(tile / tiles_x) * 4 + (lane >> 3);
+        const int2 at = tile_pixel(lane, 3);
+        const int i = (int)(tile % tiles_x) * 8 + at.x;
+        const int j = (int)(tile / tiles_x) * 4 + at.y;
         const bool inside = i < c.W && j < c.H;
         Ray ray;
         const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
