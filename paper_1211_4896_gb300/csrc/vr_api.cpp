@@ -618,6 +618,7 @@ static void free_volume(vr_volume *vol)
     if (vol->wtab) cudaFree(vol->wtab);
     if (vol->gquad) cudaFree(vol->gquad);
     if (vol->stats) cudaFree(vol->stats);
+    if (vol->median_list) cudaFree(vol->median_list);
     if (vol->brick_range) cudaFree(vol->brick_range);
     for (void *o : vol->copies)
         if (o) cudaFree(o);
@@ -1143,6 +1144,21 @@ static vr_status ensure_stats(vr_volume *vol)
     return VR_OK;
 }
 
+// Scratch of a large volume's median (its sample and list), created on first
+// use outside stream captures; NULL for a small volume or without it.
+static void *median_list(vr_volume *vol, cudaStream_t s)
+{
+    const size_t bytes = median_list_bytes((long long)vol->dims[0] * vol->dims[1] * vol->dims[2]);
+    if (!bytes || vol->median_list) return vol->median_list;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+        dev_alloc(&vol->median_list, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        vol->median_list = nullptr;
+    }
+    return vol->median_list;
+}
+
 vr_status vr_moments(vr_volume_t vol, double *dev_out, void *cuda_stream)
 {
     g_err.clear();
@@ -1167,7 +1183,14 @@ vr_status vr_histogram(vr_volume_t vol, double lo, double hi, int nbins, uint64_
     if (nbins < 1 || nbins > 16384) return invalid("nbins must be in [1, 16384]");
     if (!dev_counts || (reinterpret_cast<uintptr_t>(dev_counts) & 7u) != 0)
         return invalid("dev_counts must be non-NULL and 8-byte aligned");
-    cudaError_t e = launch_histogram(vol_dev(vol), vol->store_dtype, lo, hi, nbins,
+    // without scratch (no memory, or the stream is being captured) a slower path
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (!vol->stats && (cudaStreamIsCapturing(static_cast<cudaStream_t>(cuda_stream), &cs) != cudaSuccess ||
+                        cs != cudaStreamCaptureStatusNone || ensure_stats(vol) != VR_OK)) {
+        cudaGetLastError();
+        g_err.clear();
+    }
+    cudaError_t e = launch_histogram(vol_dev(vol), vol->store_dtype, lo, hi, nbins, vol->stats,
                                      reinterpret_cast<unsigned long long *>(dev_counts),
                                      static_cast<cudaStream_t>(cuda_stream));
     if (e != cudaSuccess) return cuda_fail(e, "vr_histogram launch");
@@ -1183,8 +1206,8 @@ vr_status vr_median(vr_volume_t vol, double *dev_median, void *cuda_stream)
         return invalid("dev_median must be non-NULL and 8-byte aligned");
     st = ensure_stats(vol);
     if (st != VR_OK) return st;
-    cudaError_t e = launch_median(vol_dev(vol), vol->store_dtype, vol->stats, dev_median,
-                                  static_cast<cudaStream_t>(cuda_stream));
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    cudaError_t e = launch_median(vol_dev(vol), vol->store_dtype, vol->stats, median_list(vol, s), dev_median, s);
     if (e != cudaSuccess) return cuda_fail(e, "vr_median launch");
     return VR_OK;
 }

@@ -110,6 +110,7 @@ struct vr_volume {
     size_t dense_bytes = 0;
     // scratch of the statistics passes (created on first use)
     void *stats = nullptr;
+    void *median_list = nullptr;        // a large volume's median: its sample and the keys near it
     // per-brick value range (min, max) for empty-space skipping (first use)
     float2 *brick_range = nullptr;
     // hardware-filter copy (created on first texture-filter render)
@@ -228,9 +229,10 @@ cudaError_t launch_forward_skip(const VolDev &v, vr_dtype dt, const CamDev &c, c
 // Global statistics (vr_stats.cu).
 size_t stats_scratch_bytes();
 cudaError_t launch_moments(const VolDev &v, vr_dtype dt, void *scratch, double *out, cudaStream_t s);
-cudaError_t launch_histogram(const VolDev &v, vr_dtype dt, double lo, double hi, int nbins,
+cudaError_t launch_histogram(const VolDev &v, vr_dtype dt, double lo, double hi, int nbins, void *scratch,
                              unsigned long long *counts, cudaStream_t s);
-cudaError_t launch_median(const VolDev &v, vr_dtype dt, void *scratch, double *median, cudaStream_t s);
+size_t median_list_bytes(long long nvox);
+cudaError_t launch_median(const VolDev &v, vr_dtype dt, void *scratch, void *list, double *median, cudaStream_t s);
 vr_status validate_job(const vr_job *job, int index);
 void purge_plans(const vr_volume *vol);
 
