@@ -722,6 +722,20 @@ struct IdentityMap {
     __device__ __forceinline__ float operator()(float v, const Cell &) const { return v; }
 };
 
+// Where a sample of the ray lies in the volume marched: at its position on the
+// ray, or, for a volume that holds part of a larger grid, that position less
+// the part's offset (exact for 0 <= off <= p).
+struct WholeGrid {
+    __device__ __forceinline__ float3 operator()(const float3 &p) const { return p; }
+};
+struct PartOfGrid {
+    float3 off;
+    __device__ __forceinline__ float3 operator()(const float3 &p) const
+    {
+        return make_float3(p.x - off.x, p.y - off.y, p.z - off.z);
+    }
+};
+
 // Whether a march leaves out the table lookup and the composite of samples
 // below z (transparent_below): the two 16-byte table loads of a sample are a
 // third of the L1 wavefronts of a brick layout's march (16-bit view of a
@@ -735,15 +749,17 @@ template <typename T, typename Map> __device__ constexpr bool skips_transparent(
 
 // One sample: composites (cur, fc) and, while the ray goes on, issues the
 // gathers of sample k + depth into (nxt, fn).
-template <typename T, int LOG2B, int L, typename Map = IdentityMap, int D = Pipeline<T>::depth>
+template <typename T, int LOG2B, int L, typename Map = IdentityMap, int D = Pipeline<T>::depth,
+          typename Place = WholeGrid>
 __device__ __forceinline__ void march_step(const VolDev &v, const ParamDev &p, const Ray &ray, int &k, bool &active,
                                            Composite &acc, const Cell &cur, const Gathered<T, L> &fc, Cell &nxt,
-                                           Gathered<T, L> &fn, float z, const Map &map = Map())
+                                           Gathered<T, L> &fn, float z, const Map &map = Map(),
+                                           const Place &place = Place())
 {
     constexpr bool N = !std::is_same<T, float>::value;
     const bool more = k + 1 < ray.n;
     if (D == 1 ? more : k + D < ray.n) {
-        nxt = locate_t<T, LOG2B, L, N>(v, sample_pos(ray, k + D, p.step));
+        nxt = locate_t<T, LOG2B, L, N>(v, place(sample_pos(ray, k + D, p.step)));
         fetch_corners<T, LOG2B, L>(v, nxt, fn);
     }
     const float val = map(interp_corners(cur, fc), cur);
@@ -761,30 +777,32 @@ __device__ __forceinline__ void march_step(const VolDev &v, const ParamDev &p, c
 }
 
 // The loop body is unrolled over depth + 1 register sets that take turns, so
-// a prefetched sample is never copied.
-template <typename T, int LOG2B, int L, typename Map = IdentityMap, int D = Pipeline<T>::depth>
+// a prefetched sample is never copied.  The march takes samples k .. ray.n - 1
+// and returns the sample after its last.
+template <typename T, int LOG2B, int L, typename Map = IdentityMap, int D = Pipeline<T>::depth,
+          typename Place = WholeGrid>
 __device__ __forceinline__ int march_ray(const VolDev &v, const ParamDev &p, const Ray &ray, bool active,
-                                         Composite &acc, float z, const Map &map = Map())
+                                         Composite &acc, float z, const Map &map = Map(), const Place &place = Place(),
+                                         int k = 0)
 {
     static_assert(D == 1 || D == 2, "pipeline depth 1 or 2");
     constexpr bool N = !std::is_same<T, float>::value;
-    int k = 0;
     Cell c0, c1, c2;
     Gathered<T, L> f0, f1, f2;
     if (active) {
-        c0 = locate_t<T, LOG2B, L, N>(v, sample_pos(ray, 0, p.step));
+        c0 = locate_t<T, LOG2B, L, N>(v, place(sample_pos(ray, k, p.step)));
         fetch_corners<T, LOG2B, L>(v, c0, f0);
-        if (D == 2 && ray.n > 1) {
-            c1 = locate_t<T, LOG2B, L, N>(v, sample_pos(ray, 1, p.step));
+        if (D == 2 && ray.n > k + 1) {
+            c1 = locate_t<T, LOG2B, L, N>(v, place(sample_pos(ray, k + 1, p.step)));
             fetch_corners<T, LOG2B, L>(v, c1, f1);
         }
     }
     if constexpr (D == 1) {
         for (;;) {
             if (!__any_sync(kFull, active)) break;
-            if (active) march_step<T, LOG2B, L, Map, D>(v, p, ray, k, active, acc, c0, f0, c1, f1, z, map);
+            if (active) march_step<T, LOG2B, L, Map, D, Place>(v, p, ray, k, active, acc, c0, f0, c1, f1, z, map, place);
             if (!__any_sync(kFull, active)) break;
-            if (active) march_step<T, LOG2B, L, Map, D>(v, p, ray, k, active, acc, c1, f1, c0, f0, z, map);
+            if (active) march_step<T, LOG2B, L, Map, D, Place>(v, p, ray, k, active, acc, c1, f1, c0, f0, z, map, place);
         }
     } else {
         // one warp vote per round of register sets (measured faster for the
@@ -792,9 +810,9 @@ __device__ __forceinline__ int march_ray(const VolDev &v, const ParamDev &p, con
         // the rest of it on its own `active`
         for (;;) {
             if (!__any_sync(kFull, active)) break;
-            if (active) march_step<T, LOG2B, L, Map, D>(v, p, ray, k, active, acc, c0, f0, c2, f2, z, map);
-            if (active) march_step<T, LOG2B, L, Map, D>(v, p, ray, k, active, acc, c1, f1, c0, f0, z, map);
-            if (active) march_step<T, LOG2B, L, Map, D>(v, p, ray, k, active, acc, c2, f2, c1, f1, z, map);
+            if (active) march_step<T, LOG2B, L, Map, D, Place>(v, p, ray, k, active, acc, c0, f0, c2, f2, z, map, place);
+            if (active) march_step<T, LOG2B, L, Map, D, Place>(v, p, ray, k, active, acc, c1, f1, c0, f0, z, map, place);
+            if (active) march_step<T, LOG2B, L, Map, D, Place>(v, p, ray, k, active, acc, c2, f2, c1, f1, z, map, place);
         }
     }
     return k;

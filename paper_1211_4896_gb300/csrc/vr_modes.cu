@@ -262,6 +262,13 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
 // sample); partial images composite over one another in depth order.
 // ---------------------------------------------------------------------------
 
+// As the plain forward (vr_forward.cu): four CTAs and two samples in flight for
+// the texture layers, the compiler's choice and the march's own depth otherwise.
+template <typename T> struct SubMinBlocks { static constexpr int value = 0; };
+template <> struct SubMinBlocks<TexLayers<float>> { static constexpr int value = 4; };
+template <typename T> struct SubDepth { static constexpr int value = Pipeline<T>::depth; };
+template <> struct SubDepth<TexLayers<float>> { static constexpr int value = 2; };
+
 // Ray parameters where the ray is inside [a, b] along one axis (intersected
 // into [s0, s1]); false when it misses.
 __device__ __forceinline__ bool slab_range(float q, float d, float a, float b, float &s0, float &s1)
@@ -292,13 +299,53 @@ __device__ __forceinline__ float eye_param(const CamDev &c, int i, int j)
     return -c.dist * sqrtf(wx * wx + wy * wy + wz * wz);
 }
 
+// The samples of a ray whose cell lies in the sub-box.  Along one axis a
+// sample's cell is clamp(floor(g), 0, n - 2), and the computed position g(k)
+// is monotone in k (fmaf of a value monotone in k), so the cell is at least lo
+// where g >= lo (everywhere if lo = 0), below hi where g < hi (everywhere if hi
+// = n - 1): the samples form one run, whose ends a bisection finds with the
+// positions the march itself computes.
+struct SubBox {
+    float3 lo, hi;             // -inf / +inf at the grid's own faces
+    __device__ __forceinline__ bool entered(const float3 &g, const float3 &d) const
+    {
+        return (d.x < 0.0f ? g.x < hi.x : g.x >= lo.x) && (d.y < 0.0f ? g.y < hi.y : g.y >= lo.y) &&
+               (d.z < 0.0f ? g.z < hi.z : g.z >= lo.z);
+    }
+    __device__ __forceinline__ bool left(const float3 &g, const float3 &d) const
+    {
+        return (d.x < 0.0f ? g.x < lo.x : g.x >= hi.x) || (d.y < 0.0f ? g.y < lo.y : g.y >= hi.y) ||
+               (d.z < 0.0f ? g.z < lo.z : g.z >= hi.z);
+    }
+    // [first, end) of the samples 0 .. r.n - 1
+    __device__ __forceinline__ int2 run(const Ray &r, float step) const
+    {
+        int a = 0, b = r.n;                          // first sample that has entered
+        while (a < b) {
+            const int m = (a + b) >> 1;
+            if (entered(sample_pos(r, m, step), r.d)) b = m; else a = m + 1;
+        }
+        const int first = a;
+        b = r.n;                                     // first sample from there that has left
+        while (a < b) {
+            const int m = (a + b) >> 1;
+            if (left(sample_pos(r, m, step), r.d)) b = m; else a = m + 1;
+        }
+        return make_int2(first, a);
+    }
+};
+
+// The samples of the run are marched as a whole render marches its rays (the
+// same pipeline and register budget), without a test per sample: eight boxes
+// of a 1080p view of the 1024^3 cube 4.18 -> 2.62 ms (the whole render of that
+// view takes 1.5; the rest is each launch's tail and 400 MB of partial images).
 template <typename T, int LOG2B, int L>
-__global__ void __launch_bounds__(kModeThreads) subbox_kernel(VolDev v, CamDev c, ParamDev p, int3 lo, int3 hi,
-                                                               int3 gdim, float3 off, float4 *partial, float *depth,
-                                                               uint32_t *count, unsigned *counter, int tiles_x,
-                                                               unsigned ntiles)
+__global__ void __launch_bounds__(kModeThreads, SubMinBlocks<T>::value) subbox_kernel(
+    VolDev v, CamDev c, ParamDev p, int3 lo, int3 hi, SubBox box, int3 gdim, float3 off, float4 *partial, float *depth,
+    uint32_t *count, unsigned *counter, int tiles_x, unsigned ntiles)
 {
     const int lane = threadIdx.x & 31;
+    const float z = skips_transparent<T, IdentityMap>() ? transparent_below(p) : 0.0f;
     for (;;) {
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
@@ -312,70 +359,25 @@ __global__ void __launch_bounds__(kModeThreads) subbox_kernel(VolDev v, CamDev c
         // rays and samples of the whole grid (gdim voxels; the camera is in its
         // coordinates); the volume holds its voxels from off on
         bool active = inside_img && setup_ray(c, gdim.x, gdim.y, gdim.z, p.step, i, j, ray);
-        // samples whose position lies in the sub-box widened by one voxel: the
-        // exact cell test below decides each of them
-        int k = 0, k_end = 0;
+        int2 run = make_int2(0, 0);
         if (active) {
+            // a ray that misses the sub-box widened by one voxel has no sample in it
             float s0 = -INFINITY, s1 = INFINITY;
-            active = slab_range(ray.q.x, ray.d.x, (float)lo.x - 1.0f, (float)hi.x + 1.0f, s0, s1) &&
-                     slab_range(ray.q.y, ray.d.y, (float)lo.y - 1.0f, (float)hi.y + 1.0f, s0, s1) &&
-                     slab_range(ray.q.z, ray.d.z, (float)lo.z - 1.0f, (float)hi.z + 1.0f, s0, s1);
-            if (active) {
-                const float k0 = floorf((s0 - ray.s_in) / p.step - 0.5f) - 1.0f;
-                const float k1 = ceilf((s1 - ray.s_in) / p.step - 0.5f) + 2.0f;
-                k = (int)fmaxf(k0, 0.0f);
-                k_end = (int)fminf(k1, (float)ray.n);
-                active = k < k_end;
-            }
+            if (slab_range(ray.q.x, ray.d.x, (float)lo.x - 1.0f, (float)hi.x + 1.0f, s0, s1) &&
+                slab_range(ray.q.y, ray.d.y, (float)lo.y - 1.0f, (float)hi.y + 1.0f, s0, s1) &&
+                slab_range(ray.q.z, ray.d.z, (float)lo.z - 1.0f, (float)hi.z + 1.0f, s0, s1))
+                run = box.run(ray, p.step);
+            active = run.x < run.y;
         }
-        float Cr = 0.0f, Cg = 0.0f, Cb = 0.0f, Tt = 1.0f;
-        int first = -1, used = 0;
-        Cell c0, c1;
-        Gathered<T, L> f0, f1;
-        auto local = [&](int q) {
-            const float3 g = sample_pos(ray, q, p.step);
-            return make_float3(g.x - off.x, g.y - off.y, g.z - off.z);     // exact for 0 <= off <= g
-        };
-        if (active) {
-            c0 = locate_t<T, LOG2B, L, false>(v, local(k));
-            fetch_corners<T, LOG2B, L>(v, c0, f0);
-        }
-        auto step = [&](const Cell &cur, const Gathered<T, L> &fc, Cell &nxt, Gathered<T, L> &fn) {
-            const bool more = k + 1 < k_end;
-            if (more) {
-                nxt = locate_t<T, LOG2B, L, false>(v, local(k + 1));
-                fetch_corners<T, LOG2B, L>(v, nxt, fn);
-            }
-            // the sample's cell in the whole grid, clamped as the whole render clamps it
-            // (x0 + fx is the local position exactly)
-            const int gx = min(max(__float2int_rd((float)cur.x0 + cur.fx) + (int)off.x, 0), gdim.x - 2);
-            const int gy = min(max(__float2int_rd((float)cur.y0 + cur.fy) + (int)off.y, 0), gdim.y - 2);
-            const int gz = min(max(__float2int_rd((float)cur.z0 + cur.fz) + (int)off.z, 0), gdim.z - 2);
-            if (gx >= lo.x && gx < hi.x && gy >= lo.y && gy < hi.y && gz >= lo.z && gz < hi.z) {
-                TfPos tp;
-                const float4 e = tf_lookup_l1(p, interp_corners(cur, fc), tp);
-                const float aT = e.w * Tt;
-                Cr = fmaf(aT, e.x, Cr);
-                Cg = fmaf(aT, e.y, Cg);
-                Cb = fmaf(aT, e.z, Cb);
-                Tt = fmaf(-e.w, Tt, Tt);
-                if (first < 0) first = k;
-                ++used;
-            }
-            ++k;
-            if (!more) active = false;
-        };
-        for (;;) {
-            if (!__any_sync(kFull, active)) break;
-            if (active) step(c0, f0, c1, f1);
-            if (!__any_sync(kFull, active)) break;
-            if (active) step(c1, f1, c0, f0);
-        }
+        Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
+        ray.n = run.y;
+        march_ray<T, LOG2B, L, IdentityMap, SubDepth<T>::value, PartOfGrid>(v, p, ray, active, acc, z, IdentityMap(),
+                                                                            PartOfGrid{off}, run.x);
         if (!inside_img) continue;
         const long long px = (long long)j * c.W + i;
-        partial[px] = make_float4(Cr, Cg, Cb, Tt);
-        depth[px] = first >= 0 ? fmaf((float)first + 0.5f, p.step, ray.s_in) - eye_param(c, i, j) : INFINITY;
-        if (count) count[px] = (uint32_t)used;
+        partial[px] = make_float4(acc.r, acc.g, acc.b, acc.T);
+        depth[px] = active ? fmaf((float)run.x + 0.5f, p.step, ray.s_in) - eye_param(c, i, j) : INFINITY;
+        if (count) count[px] = (uint32_t)(run.y - run.x);
     }
 }
 
@@ -390,12 +392,20 @@ cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const P
     const int3 l3 = make_int3(lo[0], lo[1], lo[2]), h3 = make_int3(hi[0], hi[1], hi[2]);
     const int3 g3 = make_int3(gdim[0], gdim[1], gdim[2]);
     const float3 o3 = make_float3((float)off[0], (float)off[1], (float)off[2]);
+    SubBox box;
+    float *blo = &box.lo.x, *bhi = &box.hi.x;
+    for (int a = 0; a < 3; ++a) {
+        blo[a] = lo[a] <= 0 ? -INFINITY : (float)lo[a];
+        bhi[a] = hi[a] >= gdim[a] - 1 ? INFINITY : (float)hi[a];
+    }
+    ParamDev q = p;
+    q.t_stop = -INFINITY;                       // no early termination inside a sub-box
     return visit_layout_tex(
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
             auto fn = subbox_kernel<typename Y::type, Y::log2b, Y::order>;
-            fn<<<persistent_grid(fn, ntiles), kModeThreads, 0, s>>>(v, c, p, l3, h3, g3, o3, partial, depth, count,
+            fn<<<persistent_grid(fn, ntiles), kModeThreads, 0, s>>>(v, c, q, l3, h3, box, g3, o3, partial, depth, count,
                                                                     counter, tiles_x, ntiles);
             return cudaGetLastError();
         },
