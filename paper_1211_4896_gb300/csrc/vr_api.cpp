@@ -350,6 +350,26 @@ static double ray_pitch_voxels(const vr_volume *vol, const vr_camera *cam, const
     return pitch * std::sqrt(q);
 }
 
+// Ray pitch in voxels from which a view counts as sparse: its rays share no
+// sectors (VR_SPARSE_MIN_PITCH).
+static double sparse_min_pitch()
+{
+    static const double p = [] {
+        const char *e = std::getenv("VR_SPARSE_MIN_PITCH");
+        return e ? std::atof(e) : 3.0;
+    }();
+    return p;
+}
+
+static bool sparse_view(const vr_volume *vol, const vr_camera *cam)
+{
+    double r[3];
+    cross3(cam->forward, cam->up, r);
+    const double rl = std::sqrt(dot3(r, r));
+    for (double &x : r) x /= rl;
+    return ray_pitch_voxels(vol, cam, r) >= sparse_min_pitch();
+}
+
 // Brick copy for a camera.  Its fastest axis is the one along which the
 // image's horizontal direction (in voxel units) is longest, so that a warp's
 // row of eight rays reads neighbouring elements; a view along x reads the
@@ -375,10 +395,7 @@ int preferred_copy(vr_volume *vol, const vr_camera *cam, bool may_build, cudaStr
         const char *e = std::getenv("VR_PAIRED_MAX_PITCH");
         return e ? std::atof(e) : 3.0;
     }();
-    static const double sparse_pitch = [] {
-        const char *e = std::getenv("VR_SPARSE_MIN_PITCH");
-        return e ? std::atof(e) : 3.0;
-    }();
+    const double sparse_pitch = sparse_min_pitch();
     // layout of sparse views (VR_SPARSE_LAYOUT): 'b' blocked copies (forward
     // kernels only), 'i' as dense views (rows along the image's horizontal
     // axis); default 'b' for 16-bit storage in bricks smaller than 64^3 and
@@ -884,7 +901,7 @@ vr_status vr_render(vr_volume_t vol, const vr_camera *cam, const vr_params *para
                                   dev_nsamples_out, ctr, status_word(vol), s);
     } else {
         e = launch_forward(vol_dev_copy(vol, preferred_copy(vol, cam, true, s, kReadsBlocked | kReadsLayers)),
-                           vol->store_dtype, c, p,
+                           vol->store_dtype, c, p, sparse_view(vol, cam),
                            reinterpret_cast<float4 *>(dev_rgba_out), dev_nsamples_out, ctr, s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "vr_render launch");

@@ -818,6 +818,79 @@ __device__ __forceinline__ int march_ray(const VolDev &v, const ParamDev &p, con
     return k;
 }
 
+// One ray per group of G lanes (the lanes of a ray are 32 / G apart): lane g
+// of the group takes samples g, G + g, 2 G + g, ... of the ray, so that a warp
+// holds 32 / G rays and passes through them G times faster.
+// The G samples of a round are then composited one after another by every
+// lane of the group (the same operations in the same order as march_ray, so
+// the same bits), each sample handed over by shuffles; a round whose samples
+// all lie in the table's transparent range z composites nothing.  Returns the
+// ray's sample count and acc on every lane of its group.
+template <typename T, int LOG2B, int L, int G>
+__device__ __forceinline__ int march_group(const VolDev &v, const ParamDev &p, const Ray &ray, bool hit, Composite &acc,
+                                           float z)
+{
+    constexpr bool N = !std::is_same<T, float>::value;
+    constexpr int RW = 32 / G;                               // rays per warp
+    const int lane = threadIdx.x & 31, r = lane & (RW - 1);
+    const int n = hit ? ray.n : 0;
+    int kb = 0, k = lane / RW, used = n;                     // first sample of the round, this lane's sample
+    bool live = n > 0;
+    Cell c0, c1;
+    Gathered<T, L> f0, f1;
+    auto fetch = [&](int q, Cell &c, Gathered<T, L> &f) {
+        if (live && q < n) {
+            c = locate_t<T, LOG2B, L, N>(v, sample_pos(ray, q, p.step));
+            fetch_corners<T, LOG2B, L>(v, c, f);
+        }
+    };
+    auto round = [&](const Cell &cur, const Gathered<T, L> &fc, Cell &nxt, Gathered<T, L> &fn) {
+        fetch(k + G, nxt, fn);                               // the next round's gathers
+        float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool opaque = false;
+        if (live && k < n) {
+            const float val = interp_corners(cur, fc);
+            const float u = fmaf(val, p.su, p.ou);
+            opaque = !(u < z);
+            if (opaque) {
+                TfPos tp;
+                e = tf_lookup_l1(p, val, tp);
+            }
+        }
+        const unsigned any = __ballot_sync(kFull, opaque);
+        if (any) {
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const unsigned m = (any >> (g * RW)) & ((1u << RW) - 1u);
+                if (m == 0) continue;
+                const int src = g * RW + r;
+                const float ex = __shfl_sync(kFull, e.x, src), ey = __shfl_sync(kFull, e.y, src),
+                            ez = __shfl_sync(kFull, e.z, src), ew = __shfl_sync(kFull, e.w, src);
+                if (live && ((m >> r) & 1u)) {
+                    const float aT = ew * acc.T;
+                    acc.r = fmaf(aT, ex, acc.r);
+                    acc.g = fmaf(aT, ey, acc.g);
+                    acc.b = fmaf(aT, ez, acc.b);
+                    acc.T = fmaf(-ew, acc.T, acc.T);
+                    if (acc.T <= p.t_stop) {
+                        live = false;
+                        used = kb + g + 1;
+                    }
+                }
+            }
+        }
+        kb += G;
+        k += G;
+        if (kb >= n) live = false;
+    };
+    fetch(k, c0, f0);
+    while (__any_sync(kFull, live)) {                        // two register sets in turn
+        round(c0, f0, c1, f1);
+        round(c1, f1, c0, f0);
+    }
+    return used;
+}
+
 __device__ __forceinline__ void write_pixel(const ParamDev &p, const Composite &acc, int used, float4 *out,
                                             uint32_t *nsamples, long long px)
 {

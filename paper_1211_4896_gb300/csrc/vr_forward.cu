@@ -56,6 +56,44 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
     }
 }
 
+// Sparse views (rays three or more voxels apart at the volume centre): eight
+// lanes to a ray (march_group).  Neighbouring rays share no sectors there, and
+// with a ray to each lane the lines it fetched were evicted before its next
+// samples came to use them: 59 DRAM bytes a sample against 17 compulsory, the
+// march waiting on memory 12 of 13 issue slots.  Eight consecutive samples of
+// a ray in one warp instruction use a line at once, and an eighth of the rays
+// are in flight.  1080p-like views of big cubes, rays 6 voxels apart: 2048 x
+// 2048 x 1024 float in 64^3 bricks 3.23 -> 2.33 ms, 1024 x 1024 x 700 float along
+// z 618 -> 391 us, along x 851 -> 414, tilted with an opaque table 492 -> 330;
+// float16 on blocked copies 685 -> 300 us.  Sixteen lanes gain 5-10% more
+// where rays are long and transparent and lose 15% where they end after 50
+// samples; two rounds of gathers in flight are the same trade.
+constexpr int kGroup = 8;
+
+template <typename T, int LOG2B, int L>
+__global__ void __launch_bounds__(kFwdThreads, 3) fwd_group_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
+                                                                uint32_t *nsamples, unsigned *counter, int tiles_x,
+                                                                unsigned ntiles)
+{
+    constexpr int RW = 32 / kGroup;                           // rays per warp: 2 x 2 pixels
+    const int lane = threadIdx.x & 31, r = lane & (RW - 1);
+    const float z = transparent_below(p);
+    for (;;) {
+        unsigned tile = 0;
+        if (lane == 0) tile = atomicAdd(counter, 1u);
+        tile = __shfl_sync(kFull, tile, 0);
+        if (tile >= ntiles) break;
+        const int i = (int)(tile % tiles_x) * 2 + (r & 1);
+        const int j = (int)(tile / tiles_x) * 2 + (r >> 1);
+        const bool inside = i < c.W && j < c.H;
+        Ray ray;
+        const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
+        Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
+        const int used = march_group<T, LOG2B, L, kGroup>(v, p, ray, hit, acc, z);
+        if (inside && lane < RW) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
+    }
+}
+
 // Hardware-filter alternative: tex3D with cudaFilterModeLinear (texel
 // centres at +0.5 in unnormalised coordinates).  Same camera, lookup and
 // compositing; only the interpolation differs (8-bit fractional weights).
@@ -130,14 +168,36 @@ static int fwd_ctas_per_sm(const void *fn, int cap)
     return (want > 0 && want < occ) ? want : occ;
 }
 
-// CTAs per SM for the float brick layouts, which serve the views whose rays
-// are too far apart for texture layers: three, where each resident ray keeps
-// its own cache lines live and more of them thrash L1 and L2 (four 1080p
-// views of the 4096 x 4096 x 1024 cube: along z 6.20 -> 5.45 ms, along x
-// 7.19 -> 7.01 ms; two were slower again).  The other layouts: the occupancy
-// limit (16-bit blocked copies measured the same at two, three and four).
+// CTAs per SM for the float brick layouts with a ray to each lane (dense views
+// that cannot have texture layers): three, where each resident ray keeps its
+// own cache lines live and more of them thrash L1 and L2.  The other layouts:
+// the occupancy limit.
 template <typename T> struct FwdCtaCap { static constexpr int value = 0; };
 template <> struct FwdCtaCap<float> { static constexpr int value = 3; };
+
+// Persistent grid of `tiles` tiles: per_sm CTAs on each SM, no more than
+// there are tiles for.
+static unsigned fwd_grid(int per_sm, unsigned tiles)
+{
+    const unsigned grid = (unsigned)(per_sm * sm_count()), useful = (tiles + kFwdThreads / 32 - 1) / (kFwdThreads / 32);
+    return grid < useful ? grid : (useful ? useful : 1u);
+}
+
+template <typename T, int LOG2B, int L>
+static cudaError_t launch_group_t(const VolDev &v, const CamDev &c, const ParamDev &p, float4 *out,
+                                  uint32_t *nsamples, unsigned *counter, cudaStream_t s)
+{
+    const int tiles_x = (c.W + 1) / 2, tiles_y = (c.H + 1) / 2;
+    const unsigned ntiles = (unsigned)tiles_x * (unsigned)tiles_y;
+    auto fn = fwd_group_kernel<T, LOG2B, L>;
+    const unsigned grid = fwd_grid(occupancy_blocks((const void *)fn, kFwdThreads, 0), ntiles);
+    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
+    if (e != cudaSuccess) return e;
+    log_line("forward %dx%d: layout order %d%s, %u tiles of 2x2 rays, %d lanes to a ray, grid %u x %d threads", c.W, c.H,
+             v.order, v.paired == 2 ? " blocked" : "", ntiles, kGroup, grid, kFwdThreads);
+    fn<<<grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, tiles_x, ntiles);
+    return cudaGetLastError();
+}
 
 template <typename T, int LOG2B, int L>
 static cudaError_t launch_fwd_t(const VolDev &v, const CamDev &c, const ParamDev &p, float4 *out,
@@ -147,10 +207,7 @@ static cudaError_t launch_fwd_t(const VolDev &v, const CamDev &c, const ParamDev
     const unsigned ntiles = (unsigned)tiles_x * (unsigned)tiles_y;
     auto fn = fwd_kernel<T, LOG2B, L>;
     const int per_sm = fwd_ctas_per_sm((const void *)fn, FwdCtaCap<T>::value);
-    unsigned grid = (unsigned)(per_sm * sm_count());
-    const unsigned max_useful = (ntiles + kFwdThreads / 32 - 1) / (kFwdThreads / 32);
-    if (grid > max_useful) grid = max_useful;
-    if (grid < 1) grid = 1;
+    const unsigned grid = fwd_grid(per_sm, ntiles);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     log_line("forward %dx%d: layout order %d%s, %u tiles of 8x4 rays, grid %u x %d threads (%d per SM)", c.W, c.H,
@@ -161,13 +218,18 @@ static cudaError_t launch_fwd_t(const VolDev &v, const CamDev &c, const ParamDev
     return cudaGetLastError();
 }
 
-cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, float4 *out,
+// sparse: the view's rays are too far apart to share sectors (they read the
+// bricks, their row copies or blocked copies).
+cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool sparse, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s)
 {
     return visit_layout_all(
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
+            if constexpr (!is_layers<typename Y::type>::value && !is_pair<typename Y::type>::value)
+                if (sparse)
+                    return launch_group_t<typename Y::type, Y::log2b, Y::order>(v, c, p, out, nsamples, counter, s);
             return launch_fwd_t<typename Y::type, Y::log2b, Y::order>(v, c, p, out, nsamples, counter, s);
         },
         cudaErrorInvalidValue);
@@ -179,9 +241,7 @@ cudaError_t launch_forward_texture(const vr_volume *vol, const CamDev &c, const 
     const int tiles_x = (c.W + 7) / 8, tiles_y = (c.H + 3) / 4;
     const unsigned ntiles = (unsigned)tiles_x * (unsigned)tiles_y;
     const int per_sm = occupancy_blocks((const void *)fwd_tex_kernel, kFwdThreads, 0);
-    unsigned grid = (unsigned)(per_sm * sm_count());
-    const unsigned max_useful = (ntiles + kFwdThreads / 32 - 1) / (kFwdThreads / 32);
-    if (grid > max_useful) grid = max_useful;
+    const unsigned grid = fwd_grid(per_sm, ntiles);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     fwd_tex_kernel<<<grid, kFwdThreads, 0, s>>>(vol->tex, (int)vol->dims[0], (int)vol->dims[1], (int)vol->dims[2],

@@ -1,0 +1,39 @@
+"""Sparse views march eight lanes to a ray: images and sample counts bit for
+bit those of the staged march (one ray to a lane), for rays of fewer samples
+than lanes and of many, image edges that cut the 2 x 2 tiles, early
+termination at every place in a round, opaque and transparent tables, all
+storage types and brick sizes (bricks, row copies and blocked copies)."""
+import pytest
+
+import synth
+from tests.helpers import cuda_or_skip
+
+pytestmark = pytest.mark.gpu
+DIMS = (50, 43, 61)
+
+
+@pytest.fixture(scope="module")
+def torch():
+    return cuda_or_skip()
+
+
+@pytest.mark.parametrize("store,brick", [("f32", 16), ("f32", 64), ("f16", 16), ("bf16", 32), ("f16", 64)])
+def test_groups_match_single_lanes(torch, store, brick):
+    import paper_1211_4896_gb300 as P
+    from paper_1211_4896_gb300 import _lib as L
+    vol = P.Volume(synth.hi_cube(DIMS, n_blobs=9, n_disks=0, seed=4).cuda(), store, brick=brick)
+    tables = [torch.from_numpy(t).cuda() for t in (synth.tf_ramp(256), synth.tf_random_pwl(seed=6, alpha_max=0.5))]
+    c = [0.5 * (d - 1) for d in DIMS]
+    try:
+        for q, (f, up) in enumerate((((0, 0, 1), (0, 1, 0)), ((1, 0, 0), (0, 1, 0)), ((0, -1, 0), (1, 0, 0)),
+                                     ((0.6, -0.5, 0.62), (0, 1, 0)))):
+            eye = tuple(c[a] - 150.0 * f[a] for a in range(3))
+            w, h = ((13, 9), (8, 11), (15, 14), (1, 2))[q]
+            for cam in (synth.camera_ortho(eye, f, up, 70.0, w, h), synth.camera_persp(eye, f, up, 30.0, w, h)):
+                for step, ert in ((0.31, 2.0), (0.5, 0.6), (0.5, 0.99), (9.0, 2.0), (40.0, 0.3)):
+                    for tf in tables:
+                        a, na = P.render(vol, cam, tf, -3.0, 30.0, step, ert)
+                        b, nb = P.render(vol, cam, tf, -3.0, 30.0, step, ert, filter=L.VR_FILTER_SOFTWARE_STAGED)
+                        assert torch.equal(na, nb) and torch.equal(a, b)
+    finally:
+        vol.close()
