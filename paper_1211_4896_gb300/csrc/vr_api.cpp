@@ -361,13 +361,49 @@ static double sparse_min_pitch()
     return p;
 }
 
-static bool sparse_view(const vr_volume *vol, const vr_camera *cam)
+// Pixels of the rectangle around the box's eight corners on the image (all of
+// them when a corner is not in front of a perspective eye).
+static double covered_pixels(const vr_volume *vol, const vr_camera *cam)
+{
+    double f[3], r[3], u[3];
+    const double fl = std::sqrt(dot3(cam->forward, cam->forward));
+    for (int a = 0; a < 3; ++a) f[a] = cam->forward[a] / fl;
+    cross3(f, cam->up, r);
+    const double rl = std::sqrt(dot3(r, r));
+    for (double &x : r) x /= rl;
+    cross3(r, f, u);
+    const double W = cam->width, H = cam->height;
+    double lo[2] = {W, H}, hi[2] = {0.0, 0.0};
+    for (int q = 0; q < 8; ++q) {
+        double d[3];
+        for (int a = 0; a < 3; ++a)
+            d[a] = vol->origin[a] + ((q >> a) & 1 ? (double)(vol->dims[a] - 1) * vol->spacing[a] : 0.0) - cam->eye[a];
+        double half = 0.5 * cam->ortho_height;                       // of the image's height at the corner
+        if (cam->kind == VR_CAMERA_PERSPECTIVE) {
+            const double depth = dot3(d, f);
+            if (!(depth > 0.0)) return W * H;
+            half = depth * std::tan(cam->fov_y_deg * M_PI / 360.0);
+        }
+        const double c[2] = {0.5 * W + 0.5 * H * dot3(d, r) / half, 0.5 * H - 0.5 * H * dot3(d, u) / half};
+        for (int a = 0; a < 2; ++a) {
+            lo[a] = std::fmin(lo[a], std::fmax(c[a], 0.0));
+            hi[a] = std::fmax(hi[a], std::fmin(c[a], a ? H : W));
+        }
+    }
+    return std::fmax(hi[0] - lo[0], 0.0) * std::fmax(hi[1] - lo[1], 0.0);
+}
+
+// Whether a view is marched with several lanes to a ray: its rays share no
+// sectors, or it covers fewer than eight tiles of 32 rays an SM (the figures
+// stand at fwd_group_kernel).
+static bool march_in_groups(const vr_volume *vol, const vr_camera *cam)
 {
     double r[3];
     cross3(cam->forward, cam->up, r);
     const double rl = std::sqrt(dot3(r, r));
     for (double &x : r) x /= rl;
-    return ray_pitch_voxels(vol, cam, r) >= sparse_min_pitch();
+    return ray_pitch_voxels(vol, cam, r) >= sparse_min_pitch() ||
+           covered_pixels(vol, cam) < 8.0 * 32.0 * (double)sm_count();
 }
 
 // Brick copy for a camera.  Its fastest axis is the one along which the
@@ -901,7 +937,7 @@ vr_status vr_render(vr_volume_t vol, const vr_camera *cam, const vr_params *para
                                   dev_nsamples_out, ctr, status_word(vol), s);
     } else {
         e = launch_forward(vol_dev_copy(vol, preferred_copy(vol, cam, true, s, kReadsBlocked | kReadsLayers)),
-                           vol->store_dtype, c, p, sparse_view(vol, cam),
+                           vol->store_dtype, c, p, march_in_groups(vol, cam),
                            reinterpret_cast<float4 *>(dev_rgba_out), dev_nsamples_out, ctr, s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "vr_render launch");

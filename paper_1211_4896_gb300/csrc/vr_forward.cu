@@ -56,8 +56,9 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
     }
 }
 
-// Sparse views (rays three or more voxels apart at the volume centre): eight
-// lanes to a ray (march_group).  Neighbouring rays share no sectors there, and
+// Eight lanes to a ray (march_group), for two kinds of views:
+//
+// Sparse views (rays three or more voxels apart at the volume centre).  Neighbouring rays share no sectors there, and
 // with a ray to each lane the lines it fetched were evicted before its next
 // samples came to use them: 59 DRAM bytes a sample against 17 compulsory, the
 // march waiting on memory 12 of 13 issue slots.  Eight consecutive samples of
@@ -68,6 +69,14 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
 // float16 on blocked copies 685 -> 300 us.  Sixteen lanes gain 5-10% more
 // where rays are long and transparent and lose 15% where they end after 50
 // samples; two rounds of gathers in flight are the same trade.
+//
+// Views whose volume covers few pixels (fewer than eight 8 x 4 tiles an SM):
+// with a ray to each lane they leave the SMs a few warps each, which wait out
+// every gather's latency along the whole ray.  128 x 120 x 140 cube, 320 x 200
+// pixels: float 94 -> 40 us, opaque table 83 -> 57, float16 87 -> 40.  With
+// more tiles the composite's shuffles cost more than the latency: 400 x 320
+// pixels 105 -> 60, but with the opaque table 94 -> 104; a face-on 256 x 256
+// view of a 128^3 cube, all of it covered, 82 -> 87.
 constexpr int kGroup = 8;
 
 template <typename T, int LOG2B, int L>
@@ -175,6 +184,12 @@ static int fwd_ctas_per_sm(const void *fn, int cap)
 template <typename T> struct FwdCtaCap { static constexpr int value = 0; };
 template <> struct FwdCtaCap<float> { static constexpr int value = 3; };
 
+static const char *layout_name(const VolDev &v)
+{
+    const char *names[4] = {"", " paired", " blocked", " texture layers"};
+    return names[v.paired & 3];
+}
+
 // Persistent grid of `tiles` tiles: per_sm CTAs on each SM, no more than
 // there are tiles for.
 static unsigned fwd_grid(int per_sm, unsigned tiles)
@@ -194,7 +209,7 @@ static cudaError_t launch_group_t(const VolDev &v, const CamDev &c, const ParamD
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     log_line("forward %dx%d: layout order %d%s, %u tiles of 2x2 rays, %d lanes to a ray, grid %u x %d threads", c.W, c.H,
-             v.order, v.paired == 2 ? " blocked" : "", ntiles, kGroup, grid, kFwdThreads);
+             v.order, layout_name(v), ntiles, kGroup, grid, kFwdThreads);
     fn<<<grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, tiles_x, ntiles);
     return cudaGetLastError();
 }
@@ -211,24 +226,20 @@ static cudaError_t launch_fwd_t(const VolDev &v, const CamDev &c, const ParamDev
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     log_line("forward %dx%d: layout order %d%s, %u tiles of 8x4 rays, grid %u x %d threads (%d per SM)", c.W, c.H,
-             v.order, v.paired == 1 ? " paired" : (v.paired == 2 ? " blocked" : (v.paired == 3 ? " texture layers" : "")),
-             ntiles, grid, kFwdThreads,
-             per_sm);
+             v.order, layout_name(v), ntiles, grid, kFwdThreads, per_sm);
     fn<<<grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, tiles_x, ntiles);
     return cudaGetLastError();
 }
 
-// sparse: the view's rays are too far apart to share sectors (they read the
-// bricks, their row copies or blocked copies).
-cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool sparse, float4 *out,
+// groups: eight lanes to a ray (march_in_groups).
+cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s)
 {
     return visit_layout_all(
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
-            if constexpr (!is_layers<typename Y::type>::value && !is_pair<typename Y::type>::value)
-                if (sparse)
+                if (groups)
                     return launch_group_t<typename Y::type, Y::log2b, Y::order>(v, c, p, out, nsamples, counter, s);
             return launch_fwd_t<typename Y::type, Y::log2b, Y::order>(v, c, p, out, nsamples, counter, s);
         },

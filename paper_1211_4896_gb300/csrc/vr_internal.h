@@ -145,7 +145,7 @@ int sm_count();
 cudaError_t launch_brick(const void *src, vr_dtype src_dtype, vr_volume *vol, cudaStream_t s);
 cudaError_t launch_rebrick(const vr_volume *src, vr_volume *dst, cudaStream_t s);   // same dims and storage
 vr_status build_texture(vr_volume *vol, cudaStream_t s);
-cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool sparse, float4 *out,
+cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s);
 cudaError_t launch_forward_texture(const vr_volume *vol, const CamDev &c, const ParamDev &p, float4 *out,
                                    uint32_t *nsamples, unsigned *counter, cudaStream_t s);

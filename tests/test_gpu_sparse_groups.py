@@ -1,8 +1,9 @@
-"""Sparse views march eight lanes to a ray: images and sample counts bit for
+"""Sparse views and views that cover few pixels march eight lanes to a ray: images and sample counts bit for
 bit those of the staged march (one ray to a lane), for rays of fewer samples
 than lanes and of many, image edges that cut the 2 x 2 tiles, early
 termination at every place in a round, opaque and transparent tables, all
-storage types and brick sizes (bricks, row copies and blocked copies)."""
+storage types and brick sizes (bricks, row copies and blocked copies;
+texture layers and paired copies)."""
 import pytest
 
 import synth
@@ -35,5 +36,30 @@ def test_groups_match_single_lanes(torch, store, brick):
                         a, na = P.render(vol, cam, tf, -3.0, 30.0, step, ert)
                         b, nb = P.render(vol, cam, tf, -3.0, 30.0, step, ert, filter=L.VR_FILTER_SOFTWARE_STAGED)
                         assert torch.equal(na, nb) and torch.equal(a, b)
+    finally:
+        vol.close()
+
+
+@pytest.mark.parametrize("store", ["f32", "f16", "bf16"])
+def test_small_dense_views(torch, store):
+    """Dense views of a few hundred tiles: texture layers (float) and paired
+    copies; the oblique one leaves part of the image uncovered, the last has
+    the eye inside the volume."""
+    import paper_1211_4896_gb300 as P
+    from paper_1211_4896_gb300 import _lib as L
+    vol = P.Volume(synth.hi_cube(DIMS, n_blobs=9, n_disks=0, seed=4).cuda(), store)
+    tables = [torch.from_numpy(t).cuda() for t in (synth.tf_ramp(256), synth.tf_random_pwl(seed=6, alpha_max=0.5))]
+    c = [0.5 * (d - 1) for d in DIMS]
+    try:
+        cams = [synth.camera_ortho((c[0], c[1], -50.0), (0, 0, 1), (0, 1, 0), 42.0, 61, 47),
+                synth.camera_persp((c[0] - 150.0, c[1], c[2]), (1, 0, 0), (0, 0, 1), 30.0, 90, 77),
+                synth.camera_random_persp(DIMS, seed=3, width=131, height=90),
+                synth.camera_persp(tuple(c), (0.3, 0.5, -0.8), (0, 1, 0), 70.0, 65, 66)]
+        for cam in cams:
+            for step, ert in ((0.31, 2.0), (0.5, 0.6), (1.0, 0.99)):
+                for tf in tables:
+                    a, na = P.render(vol, cam, tf, -3.0, 30.0, step, ert)
+                    b, nb = P.render(vol, cam, tf, -3.0, 30.0, step, ert, filter=L.VR_FILTER_SOFTWARE_STAGED)
+                    assert torch.equal(na, nb) and torch.equal(a, b)
     finally:
         vol.close()
