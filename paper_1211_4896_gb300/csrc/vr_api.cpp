@@ -393,17 +393,21 @@ static double covered_pixels(const vr_volume *vol, const vr_camera *cam)
     return std::fmax(hi[0] - lo[0], 0.0) * std::fmax(hi[1] - lo[1], 0.0);
 }
 
-// Whether a view is marched with several lanes to a ray: its rays share no
-// sectors, or it covers fewer than eight tiles of 32 rays an SM (the figures
-// stand at fwd_group_kernel).
-static bool march_in_groups(const vr_volume *vol, const vr_camera *cam)
+bool sparse_view(const vr_volume *vol, const vr_camera *cam)
 {
     double r[3];
     cross3(cam->forward, cam->up, r);
     const double rl = std::sqrt(dot3(r, r));
     for (double &x : r) x /= rl;
-    return ray_pitch_voxels(vol, cam, r) >= sparse_min_pitch() ||
-           covered_pixels(vol, cam) < 8.0 * 32.0 * (double)sm_count();
+    return ray_pitch_voxels(vol, cam, r) >= sparse_min_pitch();
+}
+
+// Whether a view is marched with several lanes to a ray: its rays share no
+// sectors, or it covers fewer than eight tiles of 32 rays an SM (the figures
+// stand at fwd_group_kernel).
+static bool march_in_groups(const vr_volume *vol, const vr_camera *cam)
+{
+    return sparse_view(vol, cam) || covered_pixels(vol, cam) < 8.0 * 32.0 * (double)sm_count();
 }
 
 // Brick copy for a camera.  Its fastest axis is the one along which the

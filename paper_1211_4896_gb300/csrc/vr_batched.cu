@@ -4,7 +4,8 @@
 // from one global atomic queue; a tile index maps to its job by binary search
 // over the per-job tile prefix.  The launches (counter reset + one kernel per
 // layout, independent of one another) form a CUDA graph built once and
-// replayed while the job list is unchanged.
+// replayed while the job list is unchanged; the graph of large jobs holds one
+// single-view kernel per job instead (kNodeMinTiles).
 #include "vr_device.cuh"
 
 #include <algorithm>
@@ -137,13 +138,31 @@ struct Segment {
     unsigned grid = 0;
 };
 
+// Graphs (default options) of float jobs with this many 8 x 4 tiles on
+// average, or of which half are sparse views, hold one single-view forward
+// kernel per job, all after the counter reset and independent of one another:
+// a view's CTAs take the slots that the view before it leaves at its end, as
+// the tiles of the common queue do; its camera, table and volume are kernel
+// parameters (constant operands), where the batched kernel loads its job's
+// into registers and spills; texture layers keep two samples in flight, and
+// sparse views march in groups.  Common queue -> kernels: 16 float cubes of 64
+// to 1024 voxels an axis at 512 to 1024 pixels 1.85 -> 1.79 ms, two 1080p views
+// of the 1024^3 cube 3.19 -> 2.92, 16 sparse 16-bit views of 100 to 200 pixels
+// 280 -> 205 us.  The common queue stays for the rest: the kernels' ends cost
+// more than they gain below (16 dense 16-bit views of 256 to 512 pixels 0.94 ->
+// 1.02 ms) and for paired 16-bit copies, whose kernels are the same (1.94).
+constexpr unsigned kNodeMinTiles = 8192;
+constexpr int kNodeMaxJobs = 256;
+
 // A prepared batch: job descriptors resident on the device, a work counter,
 // and (optionally) the instantiated graph of one launch.
 struct BatchPlan {
     std::vector<unsigned char> key;
     std::vector<const vr_volume *> vols;   // the volumes its jobs read (dropped with any of them)
     JobDev *djobs = nullptr;
-    unsigned *counter = nullptr;       // one work counter per group
+    unsigned *counter = nullptr;       // one work counter per group, or (nodes) per job
+    std::vector<JobDev> nodes;         // the jobs of a graph of single-view kernels, most expensive first
+    std::vector<bool> sparse;          // sparse_view of each
     int njobs = 0;
     Segment seg[kGroups];
     int log2_tw = 3;
@@ -167,8 +186,8 @@ template <typename V> static void key_put(std::vector<unsigned char> &k, const V
     k.insert(k.end(), b, b + sizeof(V));
 }
 
-static std::vector<unsigned char> plan_key(int dev, cudaStream_t s, int tile_w, int ctas, int wpt, const vr_job *jobs,
-                                           int n)
+static std::vector<unsigned char> plan_key(int dev, cudaStream_t s, int tile_w, int ctas, int wpt, bool graph,
+                                           const vr_job *jobs, int n)
 {
     std::vector<unsigned char> k;
     k.reserve(64 + (size_t)n * 200);
@@ -177,6 +196,7 @@ static std::vector<unsigned char> plan_key(int dev, cudaStream_t s, int tile_w, 
     key_put(k, tile_w);
     key_put(k, ctas);
     key_put(k, wpt);
+    key_put(k, graph);
     for (int q = 0; q < n; ++q) {
         const vr_job &J = jobs[q];
         key_put(k, J.vol);
@@ -316,10 +336,15 @@ static cudaError_t build_graph(BatchPlan *plan)
     mp.dst = plan->counter;
     mp.value = 0;
     mp.elementSize = sizeof(unsigned);
-    mp.width = kGroups;
+    mp.width = plan->nodes.empty() ? kGroups : plan->nodes.size();
     mp.height = 1;
     e = cudaGraphAddMemsetNode(&reset, graph, nullptr, 0, &mp);
-    for (int g = 0; g < kGroups && e == cudaSuccess; ++g) {
+    for (size_t q = 0; q < plan->nodes.size() && e == cudaSuccess; ++q) {
+        const JobDev &J = plan->nodes[q];
+        e = add_forward_node(graph, reset, J.v, plan->vols[0]->store_dtype, J.c, J.p, plan->sparse[q], J.out, J.nsamples,
+                             plan->counter + q);
+    }
+    for (int g = 0; g < kGroups && e == cudaSuccess && plan->nodes.empty(); ++g) {
         const Segment &sg = plan->seg[g];
         if (!sg.njobs) continue;
         const JobDev *djobs = plan->djobs + sg.first;
@@ -415,7 +440,7 @@ extern "C" vr_status vr_render_batched(const vr_job *jobs, int n, const vr_batch
     int dev = 0;
     cudaGetDevice(&dev);
 
-    const std::vector<unsigned char> key = plan_key(dev, s, tile_w, ctas, wpt, jobs, n);
+    const std::vector<unsigned char> key = plan_key(dev, s, tile_w, ctas, wpt, use_graph != 0, jobs, n);
 
     std::lock_guard<std::mutex> g(g_plans_mu);
     BatchPlan *plan = nullptr;
@@ -440,8 +465,27 @@ extern "C" vr_status vr_render_batched(const vr_job *jobs, int n, const vr_batch
         plan->log2_tw = log2_of(tile_w);
         plan->log2_wpt = log2_of(wpt);
         plan->device = dev;
+        unsigned long long tiles = 0;
+        for (int g = 0; g < kGroups; ++g) tiles += seg[g].total_tiles;
+        int nsparse = 0;
+        for (int q = 0; q < n; ++q) nsparse += sparse_view(jobs[q].vol, &jobs[q].cam);
+        if (use_graph && tile_w == 8 && ctas == 0 && wpt == 1 && n <= kNodeMaxJobs &&
+            ((jobs[0].vol->store_dtype == VR_F32 && tiles >= (unsigned long long)n * kNodeMinTiles) || 2 * nsparse >= n)) {
+            // prepare_jobs left the jobs group by group; over all of them the most
+            // expensive first, so that cheap ones fill the end
+            std::vector<int> by_cost((size_t)n);
+            for (int q = 0; q < n; ++q) by_cost[q] = q;
+            std::stable_sort(by_cost.begin(), by_cost.end(),
+                             [&](int a, int b) { return cost[order[a]] > cost[order[b]]; });
+            for (int q : by_cost) {
+                plan->nodes.push_back(hj[q]);
+                plan->sparse.push_back(sparse_view(jobs[order[q]].vol, &jobs[order[q]].cam));
+            }
+        }
         cudaError_t e = dev_alloc(reinterpret_cast<void **>(&plan->djobs), sizeof(JobDev) * (size_t)n);
-        if (e == cudaSuccess) e = dev_alloc(reinterpret_cast<void **>(&plan->counter), kGroups * sizeof(unsigned));
+        if (e == cudaSuccess)
+            e = dev_alloc(reinterpret_cast<void **>(&plan->counter),
+                          std::max<size_t>(kGroups, plan->nodes.size()) * sizeof(unsigned));
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(plan->djobs, hj.data(), sizeof(JobDev) * (size_t)n, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -19,16 +19,22 @@
 
 namespace vr {
 
-constexpr int kFwdThreads = 256;
+// Two-warp CTAs: warps do not depend on one another, and small CTAs hand an
+// SM's slots on warp pair by warp pair at the end of a view (views that follow
+// each other in a batch's graph: 16 uneven cubes 2.04 -> 1.89 ms against
+// eight-warp CTAs).
+constexpr int kFwdThreads = 64;
+constexpr int kPerSm = 256 / kFwdThreads;            // CTAs that make eight warps
 
-// Resident CTAs the register budget is sized for, and samples whose gathers
-// are in flight ahead of the one composited: for the texture layers four
-// CTAs (64 registers) with two samples ahead (the eight 1080p views of the
-// 1024^3 cube 198.6 -> 209.3 Gsamples/s, against five CTAs at 48 registers
-// with one; the batched kernel keeps the latter, 1% faster there); the
-// compiler's choice and the march's own depth for the brick layouts.
-template <typename T> struct FwdMinBlocks { static constexpr int value = 0; };   // 0: no minimum
-template <> struct FwdMinBlocks<TexLayers<float>> { static constexpr int value = 4; };
+// Resident warps the register budget is sized for, and samples whose gathers
+// are in flight ahead of the one composited: 32 warps (64 registers) for the
+// texture layers, with two samples ahead (the eight 1080p views of the 1024^3
+// cube 198.6 -> 209.3 Gsamples/s, against 40 warps at 48 registers with one;
+// the batched kernel keeps the latter, 1% faster there), and for the paired
+// copies; 24 for the other brick layouts, with the march's own depth.
+template <typename T> struct FwdMinBlocks { static constexpr int value = 3 * kPerSm; };
+template <> struct FwdMinBlocks<TexLayers<float>> { static constexpr int value = 4 * kPerSm; };
+template <typename S> struct FwdMinBlocks<Pair<S>> { static constexpr int value = 4 * kPerSm; };
 template <typename T> struct FwdDepth { static constexpr int value = Pipeline<T>::depth; };
 template <> struct FwdDepth<TexLayers<float>> { static constexpr int value = 2; };
 
@@ -80,7 +86,7 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
 constexpr int kGroup = 8;
 
 template <typename T, int LOG2B, int L>
-__global__ void __launch_bounds__(kFwdThreads, 3) fwd_group_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
+__global__ void __launch_bounds__(kFwdThreads, 3 * kPerSm) fwd_group_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
                                                                 uint32_t *nsamples, unsigned *counter, int tiles_x,
                                                                 unsigned ntiles)
 {
@@ -178,11 +184,11 @@ static int fwd_ctas_per_sm(const void *fn, int cap)
 }
 
 // CTAs per SM for the float brick layouts with a ray to each lane (dense views
-// that cannot have texture layers): three, where each resident ray keeps its
+// that cannot have texture layers): 24 warps, where each resident ray keeps its
 // own cache lines live and more of them thrash L1 and L2.  The other layouts:
 // the occupancy limit.
 template <typename T> struct FwdCtaCap { static constexpr int value = 0; };
-template <> struct FwdCtaCap<float> { static constexpr int value = 3; };
+template <> struct FwdCtaCap<float> { static constexpr int value = 3 * kPerSm; };
 
 static const char *layout_name(const VolDev &v)
 {
@@ -198,52 +204,67 @@ static unsigned fwd_grid(int per_sm, unsigned tiles)
     return grid < useful ? grid : (useful ? useful : 1u);
 }
 
-template <typename T, int LOG2B, int L>
-static cudaError_t launch_group_t(const VolDev &v, const CamDev &c, const ParamDev &p, float4 *out,
-                                  uint32_t *nsamples, unsigned *counter, cudaStream_t s)
-{
-    const int tiles_x = (c.W + 1) / 2, tiles_y = (c.H + 1) / 2;
-    const unsigned ntiles = (unsigned)tiles_x * (unsigned)tiles_y;
-    auto fn = fwd_group_kernel<T, LOG2B, L>;
-    const unsigned grid = fwd_grid(occupancy_blocks((const void *)fn, kFwdThreads, 0), ntiles);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    log_line("forward %dx%d: layout order %d%s, %u tiles of 2x2 rays, %d lanes to a ray, grid %u x %d threads", c.W, c.H,
-             v.order, layout_name(v), ntiles, kGroup, grid, kFwdThreads);
-    fn<<<grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, tiles_x, ntiles);
-    return cudaGetLastError();
-}
+// A view's kernel and its grid.
+struct FwdLaunch {
+    void (*fn)(VolDev, CamDev, ParamDev, float4 *, uint32_t *, unsigned *, int, unsigned) = nullptr;
+    int tiles_x = 0;
+    unsigned ntiles = 0, grid = 0;
+};
 
 template <typename T, int LOG2B, int L>
-static cudaError_t launch_fwd_t(const VolDev &v, const CamDev &c, const ParamDev &p, float4 *out,
-                                uint32_t *nsamples, unsigned *counter, cudaStream_t s)
+static FwdLaunch plan_fwd_t(const VolDev &v, const CamDev &c, bool groups)
 {
-    const int tiles_x = (c.W + 7) / 8, tiles_y = (c.H + 3) / 4;
-    const unsigned ntiles = (unsigned)tiles_x * (unsigned)tiles_y;
-    auto fn = fwd_kernel<T, LOG2B, L>;
-    const int per_sm = fwd_ctas_per_sm((const void *)fn, FwdCtaCap<T>::value);
-    const unsigned grid = fwd_grid(per_sm, ntiles);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    log_line("forward %dx%d: layout order %d%s, %u tiles of 8x4 rays, grid %u x %d threads (%d per SM)", c.W, c.H,
-             v.order, layout_name(v), ntiles, grid, kFwdThreads, per_sm);
-    fn<<<grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, tiles_x, ntiles);
-    return cudaGetLastError();
+    FwdLaunch f;
+    const int tw = groups ? 2 : 8, th = groups ? 2 : 4;
+    f.tiles_x = (c.W + tw - 1) / tw;
+    f.ntiles = (unsigned)f.tiles_x * (unsigned)((c.H + th - 1) / th);
+    f.fn = groups ? fwd_group_kernel<T, LOG2B, L> : fwd_kernel<T, LOG2B, L>;
+    const int per_sm = groups ? occupancy_blocks((const void *)f.fn, kFwdThreads, 0)
+                              : fwd_ctas_per_sm((const void *)f.fn, FwdCtaCap<T>::value);
+    f.grid = fwd_grid(per_sm, f.ntiles);
+    log_line("forward %dx%d: layout order %d%s, %u tiles of %dx%d rays, %d lane(s) to a ray, grid %u x %d threads (%d per SM)",
+             c.W, c.H, v.order, layout_name(v), f.ntiles, tw, th, groups ? kGroup : 1, f.grid, kFwdThreads, per_sm);
+    return f;
+}
+
+static FwdLaunch plan_fwd(const VolDev &v, vr_dtype dt, const CamDev &c, bool groups)
+{
+    return visit_layout_all(
+        v, dt,
+        [&](auto lay) {
+            using Y = decltype(lay);
+            return plan_fwd_t<typename Y::type, Y::log2b, Y::order>(v, c, groups);
+        },
+        FwdLaunch());
 }
 
 // groups: eight lanes to a ray (march_in_groups).
 cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s)
 {
-    return visit_layout_all(
-        v, dt,
-        [&](auto lay) {
-            using Y = decltype(lay);
-                if (groups)
-                    return launch_group_t<typename Y::type, Y::log2b, Y::order>(v, c, p, out, nsamples, counter, s);
-            return launch_fwd_t<typename Y::type, Y::log2b, Y::order>(v, c, p, out, nsamples, counter, s);
-        },
-        cudaErrorInvalidValue);
+    const FwdLaunch f = plan_fwd(v, dt, c, groups);
+    if (!f.fn) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
+    if (e != cudaSuccess) return e;
+    f.fn<<<f.grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, f.tiles_x, f.ntiles);
+    return cudaGetLastError();
+}
+
+// The same view as a kernel node after `reset`, which clears its counter.
+cudaError_t add_forward_node(cudaGraph_t graph, cudaGraphNode_t reset, const VolDev &v, vr_dtype dt, const CamDev &c,
+                             const ParamDev &p, bool groups, float4 *out, uint32_t *nsamples, unsigned *counter)
+{
+    FwdLaunch f = plan_fwd(v, dt, c, groups);
+    if (!f.fn) return cudaErrorInvalidValue;
+    void *args[] = {const_cast<VolDev *>(&v), const_cast<CamDev *>(&c), const_cast<ParamDev *>(&p), &out, &nsamples,
+                    &counter, &f.tiles_x, &f.ntiles};
+    cudaKernelNodeParams kp = {};
+    kp.func = (void *)f.fn;
+    kp.gridDim = dim3(f.grid);
+    kp.blockDim = dim3(kFwdThreads);
+    kp.kernelParams = args;
+    cudaGraphNode_t node = nullptr;
+    return cudaGraphAddKernelNode(&node, graph, &reset, 1, &kp);
 }
 
 cudaError_t launch_forward_texture(const vr_volume *vol, const CamDev &c, const ParamDev &p, float4 *out,

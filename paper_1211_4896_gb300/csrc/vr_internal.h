@@ -147,6 +147,9 @@ cudaError_t launch_rebrick(const vr_volume *src, vr_volume *dst, cudaStream_t s)
 vr_status build_texture(vr_volume *vol, cudaStream_t s);
 cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s);
+cudaError_t add_forward_node(cudaGraph_t graph, cudaGraphNode_t reset, const VolDev &v, vr_dtype dt, const CamDev &c,
+                             const ParamDev &p, bool groups, float4 *out, uint32_t *nsamples, unsigned *counter);
+bool sparse_view(const vr_volume *vol, const vr_camera *cam);     // rays too far apart to share sectors
 cudaError_t launch_forward_texture(const vr_volume *vol, const CamDev &c, const ParamDev &p, float4 *out,
                                    uint32_t *nsamples, unsigned *counter, cudaStream_t s);
 // Brick copy a software-filter view reads: -1 the bricks themselves, else a
