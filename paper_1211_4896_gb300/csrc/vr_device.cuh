@@ -824,23 +824,24 @@ __device__ __forceinline__ int march_ray(const VolDev &v, const ParamDev &p, con
 // The G samples of a round are then composited one after another by every
 // lane of the group (the same operations in the same order as march_ray, so
 // the same bits), each sample handed over by shuffles; a round whose samples
-// all lie in the table's transparent range z composites nothing.  Returns the
-// ray's sample count and acc on every lane of its group.
-template <typename T, int LOG2B, int L, int G>
+// all lie in the table's transparent range z composites nothing.  Takes the
+// samples k0 .. ray.n - 1 and returns the sample after its last, and acc, on
+// every lane of the ray's group.
+template <typename T, int LOG2B, int L, int G, typename Map = IdentityMap, typename Place = WholeGrid>
 __device__ __forceinline__ int march_group(const VolDev &v, const ParamDev &p, const Ray &ray, bool hit, Composite &acc,
-                                           float z)
+                                           float z, const Map &map = Map(), const Place &place = Place(), int k0 = 0)
 {
     constexpr bool N = !std::is_same<T, float>::value;
     constexpr int RW = 32 / G;                               // rays per warp
     const int lane = threadIdx.x & 31, r = lane & (RW - 1);
     const int n = hit ? ray.n : 0;
-    int kb = 0, k = lane / RW, used = n;                     // first sample of the round, this lane's sample
-    bool live = n > 0;
+    int kb = k0, k = k0 + lane / RW, used = n;               // first sample of the round, this lane's sample
+    bool live = n > k0;
     Cell c0, c1;
     Gathered<T, L> f0, f1;
     auto fetch = [&](int q, Cell &c, Gathered<T, L> &f) {
         if (live && q < n) {
-            c = locate_t<T, LOG2B, L, N>(v, sample_pos(ray, q, p.step));
+            c = locate_t<T, LOG2B, L, N>(v, place(sample_pos(ray, q, p.step)));
             fetch_corners<T, LOG2B, L>(v, c, f);
         }
     };
@@ -849,7 +850,7 @@ __device__ __forceinline__ int march_group(const VolDev &v, const ParamDev &p, c
         float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
         bool opaque = false;
         if (live && k < n) {
-            const float val = interp_corners(cur, fc);
+            const float val = map(interp_corners(cur, fc), cur);
             const float u = fmaf(val, p.su, p.ou);
             opaque = !(u < z);
             if (opaque) {
@@ -889,6 +890,16 @@ __device__ __forceinline__ int march_group(const VolDev &v, const ParamDev &p, c
         round(c1, f1, c0, f0);
     }
     return used;
+}
+
+// Lanes to a ray of the kernels that march in groups, and the pixel of a
+// lane's ray in their 2 x 2 tiles.
+constexpr int kGroup = 8;
+
+__device__ __forceinline__ int2 group_pixel(unsigned tile, int tiles_x)
+{
+    const int r = threadIdx.x & (32 / kGroup - 1);
+    return make_int2((int)(tile % tiles_x) * 2 + (r & 1), (int)(tile / tiles_x) * 2 + (r >> 1));
 }
 
 __device__ __forceinline__ void write_pixel(const ParamDev &p, const Composite &acc, int used, float4 *out,

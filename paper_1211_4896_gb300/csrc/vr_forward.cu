@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
     }
 }
 
-// Eight lanes to a ray (march_group), for two kinds of views:
+// Eight lanes to a ray (march_group, kGroup), for two kinds of views:
 //
 // Sparse views (rays three or more voxels apart at the volume centre).  Neighbouring rays share no sectors there, and
 // with a ray to each lane the lines it fetched were evicted before its next
@@ -83,29 +83,26 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
 // more tiles the composite's shuffles cost more than the latency: 400 x 320
 // pixels 105 -> 60, but with the opaque table 94 -> 104; a face-on 256 x 256
 // view of a 128^3 cube, all of it covered, 82 -> 87.
-constexpr int kGroup = 8;
-
 template <typename T, int LOG2B, int L>
 __global__ void __launch_bounds__(kFwdThreads, 3 * kPerSm) fwd_group_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
                                                                 uint32_t *nsamples, unsigned *counter, int tiles_x,
                                                                 unsigned ntiles)
 {
-    constexpr int RW = 32 / kGroup;                           // rays per warp: 2 x 2 pixels
-    const int lane = threadIdx.x & 31, r = lane & (RW - 1);
+    const int lane = threadIdx.x & 31;
     const float z = transparent_below(p);
     for (;;) {
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
         if (tile >= ntiles) break;
-        const int i = (int)(tile % tiles_x) * 2 + (r & 1);
-        const int j = (int)(tile / tiles_x) * 2 + (r >> 1);
+        const int2 at = group_pixel(tile, tiles_x);
+        const int i = at.x, j = at.y;
         const bool inside = i < c.W && j < c.H;
         Ray ray;
         const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
         const int used = march_group<T, LOG2B, L, kGroup>(v, p, ray, hit, acc, z);
-        if (inside && lane < RW) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
+        if (inside && lane < 32 / kGroup) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
     }
 }
 

@@ -210,16 +210,17 @@ int occupancy_blocks(const void *fn, int threads, size_t smem);
 cudaError_t launch_wait_selftest(unsigned *status, cudaStream_t s);
 cudaError_t launch_bounds_selftest(unsigned *status, cudaStream_t s);
 // Other uses of the march (vr_modes.cu).
-cudaError_t launch_mip(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, float4 *out,
+cudaError_t launch_mip(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
                        uint32_t *nsamples, unsigned *counter, cudaStream_t s);
-cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const float *minimap,
+cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups,
+                         const float *minimap,
                          const int region[3], float4 *out, uint32_t *nsamples, unsigned *counter, cudaStream_t s);
 cudaError_t launch_minimap(const VolDev &v, vr_dtype dt, const int region[3], float *dev_out, cudaStream_t s);
 cudaError_t launch_profile(const VolDev &v, vr_dtype dt, const CamDev &c, float step, int i, int j, float *values,
                            unsigned max_values, unsigned *count, cudaStream_t s);
 // Sort-last sub-box render and depth-ordered composite (vr_modes.cu).
 constexpr int kMaxPartials = 64;
-cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const int lo[3],
+cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, const int lo[3],
                           const int hi[3], const int gdim[3], const int off[3], float4 *partial, float *depth,
                           uint32_t *count, unsigned *counter, cudaStream_t s);
 cudaError_t launch_composite(int k, const float *const *partials, const float *const *depths, long long npx,

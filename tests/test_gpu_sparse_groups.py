@@ -63,3 +63,33 @@ def test_small_dense_views(torch, store):
                     assert torch.equal(na, nb) and torch.equal(a, b)
     finally:
         vol.close()
+
+
+@pytest.mark.parametrize("store", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("view", range(3))
+def test_a_cut_of_an_image_marched_in_groups(torch, store, view):
+    """The middle 64 x 64 pixels of a 256 x 256 orthographic image (which has a
+    ray to a lane) are, bit for bit, the 64 x 64 image of the same rays (eight
+    lanes to a ray): composite, maximum, sigma clipping, a sub-box."""
+    import paper_1211_4896_gb300 as P
+    vol = P.Volume(synth.hi_cube(DIMS, n_blobs=9, n_disks=0, seed=4).cuda(), store)
+    c = [0.5 * (d - 1) for d in DIMS]
+    f, up = (((0, 0, 1), (0, 1, 0)), ((-1, 0, 0), (0, 0, 1)), ((0.6, -0.5, 0.62), (0, 1, 0)))[view]
+    eye = tuple(c[a] - 150.0 * f[a] for a in range(3))
+    big = synth.camera_ortho(eye, f, up, 40.0, 256, 256)
+    cut = synth.camera_ortho(eye, f, up, 10.0, 64, 64)
+    at = slice(96, 160)
+    mm = P.minimap(vol, (9, 8, 7))
+    kw = dict(mode=P.VR_MODE_SIGMA, minimap=mm, region=(9, 8, 7))
+    try:
+        for tf in [torch.from_numpy(t).cuda() for t in (synth.tf_ramp(256), synth.tf_random_pwl(seed=6, alpha_max=0.5))]:
+            for step, ert in ((0.31, 2.0), (0.7, 0.9)):
+                calls = [lambda cam: P.render(vol, cam, tf, -3.0, 30.0, step, ert),
+                         lambda cam: P.render(vol, cam, tf, -3.0, 30.0, step, mode=P.VR_MODE_MIP),
+                         lambda cam: P.render(vol, cam, tf, 0.0, 8.0, step, ert, **kw),
+                         lambda cam: P.render_subbox(vol, cam, tf, -3.0, 30.0, step, (3, 5, 7), (40, 31, 52))]
+                for call in calls:
+                    for a, b in zip(call(big), call(cut)):
+                        assert torch.equal(a[at, at], b)
+    finally:
+        vol.close()
