@@ -473,17 +473,22 @@ vr_status vr_composite(int k, const float *const *dev_partials, const float *con
  *
  * vr_moments writes 5 doubles: the count of non-NaN voxels, their mean,
  * population standard deviation, minimum and maximum (NaN without values).
- * Sums as in Section 4.2: runs of 16 values in FP32, the runs in FP64, about
- * a shift (the first voxel).
+ * Sums as in Section 4.2: runs of 16 values in FP32, the runs in compensated
+ * FP32, the threads in FP64, about a shift (the first voxel).
  *
  * vr_histogram writes nbins (1 .. 16384) uint64 counts of the values in
  * [lo, hi] (finite, hi > lo) in equal bins, the value hi in the last bin;
- * values outside are not counted (Section 4.1).
+ * values outside are not counted (Section 4.1).  Its first call on a volume
+ * makes the statistics scratch; without it (no memory, a captured stream) the
+ * counts are the same, more slowly.
  *
  * vr_median writes 1 double: the value of rank (n + 1) / 2 (integer division,
  * 1-based) among the n non-NaN voxels -- the median for odd n, the lower
  * median for even n, the rank the paper's Torben method returns (Section
- * 4.3) -- by a three-pass radix select (NaN without values).
+ * 4.3) -- by a three-pass radix select, or for 2^25 voxels and more in one
+ * pass that keeps the keys near a sampled bracket (n / 128 of them at most, in
+ * scratch made on the first call; without it, or when the bracket misses, the
+ * three passes).  NaN without values.
  * Errors: INVALID_ARG, OOM (first moments/median call), CUDA.
  * ---------------------------------------------------------------------- */
 vr_status vr_moments(vr_volume_t vol, double *dev_out, void *cuda_stream);

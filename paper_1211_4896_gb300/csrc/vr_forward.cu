@@ -167,8 +167,8 @@ int occupancy_blocks(const void *fn, int threads, size_t smem)
 }
 
 // Resident CTAs per SM for the persistent forward grid: the occupancy limit,
-// at most `cap` (0: none), or VR_FWD_CTAS_PER_SM when set (a tuning knob:
-// fewer resident warps thrash the L1 and L2 less).
+// at most `cap` (0: none), or eight warps for each VR_FWD_CTAS_PER_SM when set
+// (a tuning knob: fewer resident warps thrash the L1 and L2 less).
 static int fwd_ctas_per_sm(const void *fn, int cap)
 {
     const int occ = occupancy_blocks(fn, kFwdThreads, 0);
@@ -176,7 +176,7 @@ static int fwd_ctas_per_sm(const void *fn, int cap)
         const char *s = std::getenv("VR_FWD_CTAS_PER_SM");
         return s ? std::atoi(s) : 0;
     }();
-    const int want = env > 0 ? env : cap;
+    const int want = env > 0 ? env * kPerSm : cap;
     return (want > 0 && want < occ) ? want : occ;
 }
 
