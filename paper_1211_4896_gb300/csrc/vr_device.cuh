@@ -736,6 +736,11 @@ struct PartOfGrid {
     }
 };
 
+// The same, for a march that looks every sample up: the batched kernel, whose
+// registers are full (a job's leading run kept in one more made 16 dense
+// 16-bit views with opaque tables 1% slower).
+struct LookAllUp : IdentityMap {};
+
 // Whether a march leaves out the table lookup and the composite of samples
 // below z (transparent_below): the two 16-byte table loads of a sample are a
 // third of the L1 wavefronts of a brick layout's march (16-bit view of a
@@ -744,7 +749,7 @@ struct PartOfGrid {
 // the texture unit's return path either way, and the branch costs it 1-4%.
 template <typename T, typename Map> __device__ constexpr bool skips_transparent()
 {
-    return !is_layers<T>::value || !std::is_same<Map, IdentityMap>::value;
+    return !std::is_same<Map, LookAllUp>::value && (!is_layers<T>::value || !std::is_same<Map, IdentityMap>::value);
 }
 
 // One sample: composites (cur, fc) and, while the ray goes on, issues the
