@@ -230,18 +230,62 @@ __device__ __forceinline__ int bin64(float a, double lo, double range, int nbins
     return (int)floor(((double)a - lo) / range * (double)nbins);
 }
 
-// edge[b], 1 <= b < nbins: the least float whose bin64 is b or more, searched
-// from the float nearest to the edge (at most a few steps: the floats there
-// are 0.01 bins or less apart).
-__global__ void bin_edges_kernel(double lo, double hi, int nbins, float *edge)
+// Keys that order like the values (no NaN).
+__device__ __forceinline__ unsigned order_key(float a)
+{
+    const unsigned u = __float_as_uint(a);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+__device__ __forceinline__ float key_value(unsigned k)
+{
+    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
+// edge[b], 1 <= b < nbins: the least of the floats in [flo, fhi] whose bin64 is
+// b or more (above fhi if there is none).  bin64 never falls as the value
+// grows, so a search over the floats' keys is exact: from the float nearest to
+// the edge in doubling steps, then by bisection.  Nearly every edge takes two
+// decisions; where an edge lies at or near zero the floats are far closer
+// together than the FP64 expression can tell apart (for lo = -0.1, hi = 0.2 and
+// 30 bins it puts everything from -6.9e-18 on into bin 10), and it takes up to
+// 64.
+__global__ void bin_edges_kernel(double lo, double hi, float flo, float fhi, int nbins, float *edge)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < 1 || b >= nbins) return;
     const double range = hi - lo;
-    float a = (float)(lo + range * (double)b / (double)nbins);
-    for (int step = 0; step < 64 && bin64(a, lo, range, nbins) >= b; ++step) a = nextafterf(a, -INFINITY);
-    for (int step = 0; step < 64 && bin64(a, lo, range, nbins) < b; ++step) a = nextafterf(a, INFINITY);
-    edge[b] = a;
+    const unsigned first = order_key(flo), last = order_key(fhi);
+    auto reaches = [&](unsigned k) { return bin64(key_value(k), lo, range, nbins) >= b; };
+    const float near = (float)(lo + range * (double)b / (double)nbins);
+    // below: a key that does not reach b (or first - 1); at: one that does (or last + 1)
+    unsigned k = order_key(fminf(fmaxf(near, flo), fhi)), below = first - 1, at = last + 1;
+    if (reaches(k)) {
+        at = k;
+        for (unsigned d = 1; at > first; d = min(d, 1u << 30) * 2) {
+            k = at - first > d ? at - d : first;
+            if (!reaches(k)) {
+                below = k;
+                break;
+            }
+            at = k;
+        }
+    } else {
+        below = k;
+        for (unsigned d = 1; below < last; d = min(d, 1u << 30) * 2) {
+            k = last - below > d ? below + d : last;
+            if (reaches(k)) {
+                at = k;
+                break;
+            }
+            below = k;
+        }
+    }
+    while (at - below > 1) {
+        k = below + (at - below) / 2;
+        if (reaches(k)) at = k; else below = k;
+    }
+    edge[b] = key_value(at);
 }
 
 // With `copies` = 32 each lane of a warp counts into its own copy of the
@@ -294,17 +338,6 @@ __global__ void __launch_bounds__(kStatThreads) histogram_kernel(VolDev v, doubl
 // ---------------------------------------------------------------------------
 // Median: radix select on keys that order like the values.
 // ---------------------------------------------------------------------------
-
-__device__ __forceinline__ unsigned order_key(float a)
-{
-    const unsigned u = __float_as_uint(a);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-__device__ __forceinline__ float key_value(unsigned k)
-{
-    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
 
 // How the digits of the median's key are found: by passes over all voxels, or
 // over the list of keys that the collecting pass kept.
@@ -658,8 +691,8 @@ cudaError_t launch_histogram(const VolDev &v, vr_dtype dt, double lo, double hi,
     float *edge = nullptr;
     if (scratch && fast && (long long)v.nx * v.ny * v.nz >= kEdgesMinVoxels) {
         edge = reinterpret_cast<float *>(static_cast<unsigned char *>(scratch) + kEdgeOffset);
-        bin_edges_kernel<<<(unsigned)((nbins + kEdgeThreads - 1) / kEdgeThreads), kEdgeThreads, 0, s>>>(lo, hi, nbins,
-                                                                                               edge);
+        bin_edges_kernel<<<(unsigned)((nbins + kEdgeThreads - 1) / kEdgeThreads), kEdgeThreads, 0, s>>>(lo, hi, flo_in,
+                                                                                               fhi_in, nbins, edge);
     }
     return by_storage(v, dt, [&](auto lay) {
         using Y = decltype(lay);
