@@ -399,8 +399,9 @@ vr_status vr_render_batched_noalloc(const vr_job *jobs, int n, int tile_w, int t
  * region of an axis keeps the remainder), m[a] = ceil(dims[a] / region[a])
  * regions per axis.  Writes m0 * m1 * m2 float pairs to dev_minimap (x
  * fastest; 8-byte aligned, caller-owned): the mean and the population
- * standard deviation of the region's stored voxel values, summed in FP64
- * (two passes) and rounded to float32.  Point (i, j, k) sits at voxel
+ * standard deviation of the region's stored voxel values, from sums of two
+ * floats each (FP64 sums for regions above 2^21 voxels) and rounded to
+ * float32.  Point (i, j, k) sits at voxel
  * ((i + 1/2) region - 1/2, ...) for the interpolation of VR_MODE_SIGMA.
  * Asynchronous on cuda_stream.  Errors: INVALID_ARG, CUDA.
  * ---------------------------------------------------------------------- */

@@ -290,19 +290,28 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
 // one CTA per region.
 //
 // FP64 adds and fused multiply-adds run at two lanes per clock and SM here:
-// two passes of them took 11.9 ms for a 1024^3 float cube in regions of 32^3,
-// where reading its bricks takes 0.8 ms; this takes 2.1 ms (16^3: 15.6 -> 3.1,
-// 64^3: 12.1 -> 1.9; 300 x 331 x 290 in 16 bits, 9^3: 1.15 -> 0.25), bound by
-// FP32 instructions.  So a region is read once, and its sums of
+// two passes of them take 5.1 ms for a 768^3 float cube in regions of 32^3,
+// where reading its bricks takes 0.33 ms; this takes 0.96 ms (1.55 with a NaN
+// in every region, 1.86 where every region takes the second pass below), bound
+// by FP32 instructions.  So a region is read once, and its sums of
 // d = a - shift and of d^2 (shift: the region's first voxel) are kept as
 // unevaluated sums of two floats, with the rounding errors of every
 // subtraction, product and addition carried along (Knuth's two-sum and the
-// fused product error): about 25 FP32 operations a voxel, 47 significant
-// bits.  The variance (S2 - S1^2 / n) / n is then formed in FP64; as the shift
-// is itself a voxel of the region, (shift - mean)^2 <= n var, and its relative
-// error stays below n 2^-47.  Regions that this does not cover take the two
-// FP64 passes: above 2^21 voxels, non-finite sums, or deviations whose squares
-// leave the float range.
+// fused product error): about 25 FP32 operations a voxel.  The low parts are
+// plain FP32 sums, so the two are brought back to hi + lo with |lo| below half
+// an ulp of hi every kRenorm values: each addition's error then stays below
+// 2^-25 kRenorm / 2 ulps of hi, and that of the sums of the 2^13 values that a
+// thread has at most below 2^-30 of them, if all errors pointed one way.  The
+// variance S2 / n - (S1 / n)^2 is formed in FP64 and loses what the shift is
+// away from the mean: where (S1 / n)^2 exceeds 16 variances (a first voxel four
+// deviations off: 6e-5 of the regions of noise), a second pass has the mean
+// found as its shift, and so do deviations whose squares leave the float
+// range, scaled by a power of two.  Against 64 bits, restated on the CPU over
+// noise, outliers up to 1e7 as the first voxel and quantised data in up to
+// 128^3: 1e-12 of the deviation at most (without the second pass 2.6e-6),
+// where rounding the result to float is 6e-8.
+// A region with a voxel that is not finite needs no sums; one above 2^21
+// voxels, or whose differences overflow, takes two FP64 passes.
 // ---------------------------------------------------------------------------
 
 constexpr int kMiniThreads = 256;                  // 64 or 128 for regions of few voxels
@@ -341,6 +350,7 @@ __device__ __forceinline__ float brick_voxel(const VolDev &v, int x, int y, int 
 }
 
 // A sum kept as hi + lo, hi the rounded sum so far.
+constexpr int kRenorm = 32;
 struct TwoFloat {
     float hi = 0.0f, lo = 0.0f;
     __device__ __forceinline__ void add(float x)
@@ -349,87 +359,163 @@ struct TwoFloat {
         lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b)));
         hi = s;
     }
+    __device__ __forceinline__ void renorm()
+    {
+        const float x = lo;
+        lo = 0.0f;
+        add(x);
+    }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
+// A region of voxels [x0, x0 + lx) x [y0, y0 + ly) x [z0, z0 + lz).
+struct Region {
+    int x0, y0, z0, lx, ly, lz;
+};
+
+// Calls f(value) for every voxel of the region (each thread its own) and
+// after() after every U of a thread's.
+template <typename T, typename F, typename G>
+__device__ __forceinline__ void for_region(const VolDev &v, const Region &q, F &&f, G &&after)
+{
+    const T *data = static_cast<const T *>(v.data);
+    const int B1 = (1 << v.log2b) + 1;
+    // threads: 2^bx along x, then 2^by along y, the rest along z
+    const int bx = min(q.lx > 1 ? 32 - __clz(q.lx - 1) : 0, 5);
+    const int by = min(q.ly > 1 ? 32 - __clz(q.ly - 1) : 0, 31 - __clz((int)blockDim.x) - bx);
+    const int tx = threadIdx.x & ((1 << bx) - 1), ty = (threadIdx.x >> bx) & ((1 << by) - 1);
+    const int tz = threadIdx.x >> (bx + by), sz = (int)blockDim.x >> (bx + by);
+    constexpr int U = 4;                                    // loads in flight
+    for (int x = tx; x < q.lx; x += 1 << bx) {
+        const long long ex = axis_offset(q.x0 + x, v.log2b, v.nbx, v.stride, 1);
+        for (int y = ty; y < q.ly; y += 1 << by) {
+            const T *row = data + ex + axis_offset(q.y0 + y, v.log2b, v.nby, v.stride * v.nbx, B1);
+            for (int z = tz; z < q.lz; z += U * sz) {
+                T raw[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (z + u * sz < q.lz)
+                        raw[u] = row[axis_offset(q.z0 + z + u * sz, v.log2b, v.nbz, v.stride * v.nbx * v.nby, B1 * B1)];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (z + u * sz >= q.lz) break;
+                    f(to_f(raw[u]));
+                }
+                after(U);
+            }
+        }
+    }
+}
+
+// Sums over the region of d = (a - shift) scale and d^2 (SCALED; else scale is
+// 1), and the largest |d|, on every thread of the CTA.
+struct RegionSums {
+    double s1, s2;
+    float far;
+};
+
+template <typename T, bool SCALED>
+__device__ __forceinline__ RegionSums region_sums(const VolDev &v, const Region &q, float shift, float scale, double *red)
+{
+    TwoFloat s1, s2;
+    float far = 0.0f;
+    int run = 0;
+    for_region<T>(
+        v, q,
+        [&](float a) {
+            float d = __fadd_rn(a, -shift);
+            const float b = __fadd_rn(d, -a);                                          // d + e = a - shift
+            float e = __fadd_rn(__fadd_rn(a, -__fadd_rn(d, -b)), __fadd_rn(-shift, -b));
+            if (SCALED) d = __fmul_rn(d, scale), e = __fmul_rn(e, scale);
+            const float p = __fmul_rn(d, d);
+            s1.add(d);
+            s1.lo = __fadd_rn(s1.lo, e);
+            s2.add(p);
+            s2.lo = __fadd_rn(s2.lo, __fmaf_rn(__fadd_rn(d, d), e, __fmaf_rn(d, d, -p)));
+            far = fmaxf(far, fabsf(d));
+        },
+        [&](int n) {
+            if ((run += n) >= kRenorm) {
+                s1.renorm();
+                s2.renorm();
+                run = 0;
+            }
+        });
+    RegionSums r;
+    r.s1 = block_sum(s1.value(), red);
+    r.s2 = block_sum(s2.value(), red);
+    for (int o = 16; o > 0; o >>= 1) far = fmaxf(far, __shfl_xor_sync(kFull, far, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)far;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) far = fmaxf(far, (float)red[w]);
+    r.far = far;
+    return r;
+}
+
 // The region's mean and variance by two passes in FP64.
 template <typename T>
-__device__ double2 region_two_pass(const VolDev &v, int x0, int y0, int z0, int lx, int ly, int lz, double *red)
+__device__ double2 region_two_pass(const VolDev &v, const Region &q, double *red)
 {
-    const long long cnt = (long long)lx * ly * lz;
+    const long long cnt = (long long)q.lx * q.ly * q.lz;
     double s = 0.0;
     for (long long e = threadIdx.x; e < cnt; e += blockDim.x) {
-        const int x = (int)(e % lx), y = (int)((e / lx) % ly), z = (int)(e / ((long long)lx * ly));
-        s += (double)brick_voxel<T>(v, x0 + x, y0 + y, z0 + z);
+        const int x = (int)(e % q.lx), y = (int)((e / q.lx) % q.ly), z = (int)(e / ((long long)q.lx * q.ly));
+        s += (double)brick_voxel<T>(v, q.x0 + x, q.y0 + y, q.z0 + z);
     }
     const double mean = block_sum(s, red) / (double)cnt;
     double ss = 0.0;
     for (long long e = threadIdx.x; e < cnt; e += blockDim.x) {
-        const int x = (int)(e % lx), y = (int)((e / lx) % ly), z = (int)(e / ((long long)lx * ly));
-        const double d = (double)brick_voxel<T>(v, x0 + x, y0 + y, z0 + z) - mean;
+        const int x = (int)(e % q.lx), y = (int)((e / q.lx) % q.ly), z = (int)(e / ((long long)q.lx * q.ly));
+        const double d = (double)brick_voxel<T>(v, q.x0 + x, q.y0 + y, q.z0 + z) - mean;
         ss += d * d;
     }
     return make_double2(mean, block_sum(ss, red) / (double)cnt);
 }
 
+// The region's mean and variance by the one-pass sums.
 template <typename T>
-__global__ void __launch_bounds__(kMiniThreads) minimap_kernel(VolDev v, int rx, int ry, int rz, int mx, int my,
+__device__ double2 region_one_pass(const VolDev &v, const Region &q, double *red)
+{
+    const double n = (double)((long long)q.lx * q.ly * q.lz);
+    float shift = brick_voxel<T>(v, q.x0, q.y0, q.z0);
+    RegionSums t = region_sums<T, false>(v, q, shift, 1.0f, red);
+    double m = t.s1 / n, var = t.s2 / n - m * m;
+    const bool in_range = t.far >= 1e-12f && t.far <= 1e18f;
+    if (isfinite(t.s1)) {                                       // so every voxel is finite
+        if (t.far == 0.0f || (in_range && m * m <= 16.0 * var)) return make_double2((double)shift + m, fmax(var, 0.0));
+        shift = (float)((double)shift + m);
+        const float scale = in_range ? 1.0f : ldexpf(1.0f, min(max(-ilogbf(t.far), -126), 126));
+        t = region_sums<T, true>(v, q, shift, scale, red);
+        if (isfinite(t.s1) && isfinite(t.s2)) {
+            m = t.s1 / n;
+            var = fmax(t.s2 / n - m * m, 0.0) / ((double)scale * (double)scale);
+            return make_double2((double)shift + m / (double)scale, var);
+        }
+    } else {
+        // NaN, or infinities of both signs: no mean; of one sign: that one; no deviation
+        int kinds = 0;
+        for_region<T>(v, q, [&](float a) { kinds |= a != a ? 3 : (a == INFINITY ? 1 : (a == -INFINITY ? 2 : 0)); },
+                      [](int) {});
+        const bool up = __syncthreads_or(kinds & 1), down = __syncthreads_or(kinds & 2);
+        if (up || down) return make_double2(up && down ? (double)NAN : (up ? INFINITY : -INFINITY), (double)NAN);
+    }
+    return region_two_pass<T>(v, q, red);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kMiniThreads, 4) minimap_kernel(VolDev v, int rx, int ry, int rz, int mx, int my,
                                                                float2 *out)
 {
     __shared__ double red[32];
-    const long long q = blockIdx.x;
-    const int i = (int)(q % mx), j = (int)((q / mx) % my), k = (int)(q / ((long long)mx * my));
-    const int x0 = i * rx, y0 = j * ry, z0 = k * rz;
-    const int lx = min(rx, v.nx - x0), ly = min(ry, v.ny - y0), lz = min(rz, v.nz - z0);
-    const long long cnt = (long long)lx * ly * lz;
-    double2 r = make_double2(0.0, 0.0);
-    bool covered = cnt <= kMiniMaxOnePass;                      // the same on every thread
-    if (covered) {
-        const T *data = static_cast<const T *>(v.data);
-        const int B1 = (1 << v.log2b) + 1;
-        const float shift = brick_voxel<T>(v, x0, y0, z0);
-        // threads: 2^bx along x, then 2^by along y, the rest along z
-        const int bx = min(lx > 1 ? 32 - __clz(lx - 1) : 0, 5);
-        const int by = min(ly > 1 ? 32 - __clz(ly - 1) : 0, 31 - __clz((int)blockDim.x) - bx);
-        const int tx = threadIdx.x & ((1 << bx) - 1), ty = (threadIdx.x >> bx) & ((1 << by) - 1);
-        const int tz = threadIdx.x >> (bx + by), sz = (int)blockDim.x >> (bx + by);
-        TwoFloat s1, s2;
-        float far = 0.0f;
-        constexpr int U = 4;                                    // loads in flight
-        for (int x = tx; x < lx; x += 1 << bx) {
-            const long long ex = axis_offset(x0 + x, v.log2b, v.nbx, v.stride, 1);
-            for (int y = ty; y < ly; y += 1 << by) {
-                const T *row = data + ex + axis_offset(y0 + y, v.log2b, v.nby, v.stride * v.nbx, B1);
-                for (int z = tz; z < lz; z += U * sz) {
-                    T raw[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (z + u * sz < lz)
-                            raw[u] = row[axis_offset(z0 + z + u * sz, v.log2b, v.nbz, v.stride * v.nbx * v.nby, B1 * B1)];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        if (z + u * sz >= lz) break;
-                        const float a = to_f(raw[u]);
-                        const float d = __fadd_rn(a, -shift), b = __fadd_rn(d, -a);       // d + e = a - shift
-                        const float e = __fadd_rn(__fadd_rn(a, -__fadd_rn(d, -b)), __fadd_rn(-shift, -b));
-                        const float p = __fmul_rn(d, d);
-                        s1.add(d);
-                        s1.lo = __fadd_rn(s1.lo, e);
-                        s2.add(p);
-                        s2.lo = __fadd_rn(s2.lo, __fmaf_rn(__fadd_rn(d, d), e, __fmaf_rn(d, d, -p)));
-                        far = fmaxf(far, fabsf(d));
-                    }
-                }
-            }
-        }
-        const double n = (double)cnt, t1 = block_sum(s1.value(), red), t2 = block_sum(s2.value(), red);
-        covered = isfinite(t1) && isfinite(t2) && !__syncthreads_or(far > 1e18f) &&
-                  (!__syncthreads_or(far > 0.0f) || __syncthreads_or(far > 1e-12f));
-        const double m = t1 / n;
-        r = make_double2((double)shift + m, fmax(t2 / n - m * m, 0.0));
-    }
-    if (!covered) r = region_two_pass<T>(v, x0, y0, z0, lx, ly, lz, red);
-    if (threadIdx.x == 0) out[q] = make_float2((float)r.x, (float)sqrt(r.y));
+    const long long at = blockIdx.x;
+    const int i = (int)(at % mx), j = (int)((at / mx) % my), k = (int)(at / ((long long)mx * my));
+    Region q;
+    q.x0 = i * rx, q.y0 = j * ry, q.z0 = k * rz;
+    q.lx = min(rx, v.nx - q.x0), q.ly = min(ry, v.ny - q.y0), q.lz = min(rz, v.nz - q.z0);
+    const double2 r = (long long)q.lx * q.ly * q.lz <= kMiniMaxOnePass ? region_one_pass<T>(v, q, red)
+                                                                       : region_two_pass<T>(v, q, red);
+    if (threadIdx.x == 0) out[at] = make_float2((float)r.x, (float)sqrt(r.y));
 }
 
 cudaError_t launch_minimap(const VolDev &v, vr_dtype dt, const int region[3], float *dev_out, cudaStream_t s)
