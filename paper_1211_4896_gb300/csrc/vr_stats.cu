@@ -350,7 +350,7 @@ struct SelectState {
     unsigned long long k;      // rank still to find among the values matching the prefix (1-based)
     // the collecting pass
     unsigned digit[2];         // top digits of the sample's two ranks
-    unsigned long long rank[2];
+    unsigned long long rank[2], before[2];      // the ranks within those digits, and the sample's keys before them
     unsigned key_lo, key_hi;   // the bracket
     unsigned long long count;  // keys in the bracket (those beyond the list's capacity are not in it)
     unsigned long long below;  // keys under the bracket
@@ -501,9 +501,12 @@ __global__ void __launch_bounds__(kStatThreads) sample_hist_kernel(const unsigne
     }
 }
 
-// One CTA: the digits of the sample's two ranks; after the second, the bracket.
+// One CTA: the digits of the sample's two ranks; after the second, the bracket,
+// and whether it holds at most `limit` of the sample's keys (kSelectList: the
+// voxels are collected).
 __global__ void __launch_bounds__(kSelectThreads) sample_select_kernel(int pass, SelectState *st,
-                                                                        unsigned long long *hist)
+                                                                        unsigned long long *hist,
+                                                                        unsigned long long limit)
 {
     int d[2];
     unsigned long long before[2], rank[2];
@@ -516,6 +519,7 @@ __global__ void __launch_bounds__(kSelectThreads) sample_select_kernel(int pass,
         rank[0] = st->rank[0], rank[1] = st->rank[1];
     }
     for (int r = 0; r < 2; ++r) find_rank(hist + (pass ? r * 2048 : 0), 2048, rank[r], &d[r], &before[r]);
+    const unsigned long long held = pass ? st->before[1] + before[1] + hist[2048 + d[1]] - st->before[0] - before[0] : 0ull;
     __syncthreads();
     for (int b = threadIdx.x; b < 2 * 2048; b += blockDim.x) hist[b] = 0ull;
     if (threadIdx.x != 0) return;
@@ -523,12 +527,14 @@ __global__ void __launch_bounds__(kSelectThreads) sample_select_kernel(int pass,
         if (pass == 0) {
             st->digit[r] = (unsigned)d[r];
             st->rank[r] = rank[r] - before[r];
+            st->before[r] = before[r];
         } else {
             const unsigned key = (st->digit[r] << 21) | ((unsigned)d[r] << 10);
             if (r == 0) st->key_lo = key;
             else st->key_hi = key | 1023u;
         }
     }
+    if (pass) st->mode = held <= limit ? kSelectList : kSelectVoxels;
 }
 
 // The pass over the voxels: count and below-bracket count of the non-NaN
@@ -540,6 +546,7 @@ template <typename T, int LOG2B>
 __global__ void __launch_bounds__(kStatThreads) collect_kernel(VolDev v, SelectState *st, unsigned *list, unsigned cap)
 {
     static_assert(kStatThreads * U <= kMaxFace, "the staging buffer holds a round of values");
+    if (st->mode != kSelectList) return;
     __shared__ unsigned stage[kStageCap], staged;
     __shared__ unsigned long long base;
     if (threadIdx.x == 0) staged = 0u;
@@ -587,7 +594,7 @@ __global__ void __launch_bounds__(kStatThreads) collect_kernel(VolDev v, SelectS
 __global__ void list_begin_kernel(SelectState *st, unsigned cap)
 {
     const unsigned long long k = (st->n + 1) / 2;
-    if (st->count <= cap && k > st->below && k <= st->below + st->count) {
+    if (st->mode == kSelectList && st->count <= cap && k > st->below && k <= st->below + st->count) {
         st->mode = kSelectList;
         st->k = k - st->below;
     } else {
@@ -735,10 +742,13 @@ cudaError_t launch_median(const VolDev &v, vr_dtype dt, void *scratch, void *lis
             unsigned *sample = static_cast<unsigned *>(list), *keys = sample + (1u << kSampleLog2);
             const unsigned cap = (unsigned)((long long)v.nx * v.ny * v.nz / 128);
             const unsigned grid = (unsigned)sm_count() * 4;
+            // sample places inside the cube that stand for cap voxels
+            const double cells = (double)nbricks * (double)(1LL << 3 * v.log2b);
+            const auto limit = (unsigned long long)(std::fmin(1.0, (double)v.nx * v.ny * v.nz / cells) * (1 << kSampleLog2) / 128);
             sample_kernel<T, Y::log2b><<<grid, kStatThreads, 0, s>>>(v, sample, hist);
-            sample_select_kernel<<<1, kSelectThreads, 0, s>>>(0, st, hist);
+            sample_select_kernel<<<1, kSelectThreads, 0, s>>>(0, st, hist, 0);
             sample_hist_kernel<<<grid, kStatThreads, 0, s>>>(sample, st, hist);
-            sample_select_kernel<<<1, kSelectThreads, 0, s>>>(1, st, hist);
+            sample_select_kernel<<<1, kSelectThreads, 0, s>>>(1, st, hist, limit);
             auto fn = collect_kernel<T, Y::log2b>;
             fn<<<stat_grid((const void *)fn, nbricks), kStatThreads, 0, s>>>(v, st, keys, cap);
             list_begin_kernel<<<1, 1, 0, s>>>(st, cap);
