@@ -479,9 +479,9 @@ vr_status vr_composite(int k, const float *const *dev_partials, const float *con
  *
  * vr_histogram writes nbins (1 .. 16384) uint64 counts of the values in
  * [lo, hi] (finite, hi > lo) in equal bins, the value hi in the last bin;
- * values outside are not counted (Section 4.1).  Its first call on a volume
- * makes the statistics scratch; without it (no memory, a captured stream) the
- * counts are the same, more slowly.
+ * values outside are not counted (Section 4.1).  For volumes of 2^23 voxels and
+ * more its first call makes the statistics scratch; without it (no memory, a
+ * captured stream) the counts are the same, more slowly.
  *
  * vr_median writes 1 double: the value of rank (n + 1) / 2 (integer division,
  * 1-based) among the n non-NaN voxels -- the median for odd n, the lower

@@ -1242,8 +1242,9 @@ vr_status vr_histogram(vr_volume_t vol, double lo, double hi, int nbins, uint64_
         return invalid("dev_counts must be non-NULL and 8-byte aligned");
     // without scratch (no memory, or the stream is being captured) a slower path
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (!vol->stats && (cudaStreamIsCapturing(static_cast<cudaStream_t>(cuda_stream), &cs) != cudaSuccess ||
-                        cs != cudaStreamCaptureStatusNone || ensure_stats(vol) != VR_OK)) {
+    if (!vol->stats && histogram_wants_edges((long long)vol->dims[0] * vol->dims[1] * vol->dims[2], lo, hi, nbins) &&
+        (cudaStreamIsCapturing(static_cast<cudaStream_t>(cuda_stream), &cs) != cudaSuccess ||
+         cs != cudaStreamCaptureStatusNone || ensure_stats(vol) != VR_OK)) {
         cudaGetLastError();
         g_err.clear();
     }

@@ -232,6 +232,7 @@ cudaError_t launch_forward_skip(const VolDev &v, vr_dtype dt, const CamDev &c, c
                                 unsigned *counter, cudaStream_t s);
 // Global statistics (vr_stats.cu).
 size_t stats_scratch_bytes();
+bool histogram_wants_edges(long long nvox, double lo, double hi, int nbins);      // whether it uses the scratch
 cudaError_t launch_moments(const VolDev &v, vr_dtype dt, void *scratch, double *out, cudaStream_t s);
 cudaError_t launch_histogram(const VolDev &v, vr_dtype dt, double lo, double hi, int nbins, void *scratch,
                              unsigned long long *counts, cudaStream_t s);

@@ -676,6 +676,23 @@ cudaError_t launch_moments(const VolDev &v, vr_dtype dt, void *scratch, double *
 constexpr long long kEdgesMinVoxels = 1LL << 23;
 constexpr int kEdgeThreads = 32;          // one warp a CTA: spread over the SMs' FP64 units
 
+// The error of the FP32 estimate of a bin, in bins: rounding of lo and of a - lo
+// (each within one ulp of max(|lo|, |hi|)) times the scale, plus the scale's
+// rounding.
+static double estimate_error(double lo, double hi, int nbins)
+{
+    const double m = std::fmax(std::fabs(lo), std::fabs(hi));
+    const double ulp = m > 0.0 ? std::ldexp(1.0, std::ilogb(m) - 23) : 0.0;
+    return 2.0 * ulp * (double)nbins / (hi - lo) + 4.0 * 6e-8 * (double)nbins;
+}
+
+constexpr double kFastError = 0.02;       // bins: the estimate is used up to this error
+
+bool histogram_wants_edges(long long nvox, double lo, double hi, int nbins)
+{
+    return nvox >= kEdgesMinVoxels && estimate_error(lo, hi, nbins) <= kFastError;
+}
+
 // scratch: the statistics scratch, or NULL (near an edge the bin is then
 // decided in FP64).
 cudaError_t launch_histogram(const VolDev &v, vr_dtype dt, double lo, double hi, int nbins, void *scratch,
@@ -685,18 +702,14 @@ cudaError_t launch_histogram(const VolDev &v, vr_dtype dt, double lo, double hi,
     if (e != cudaSuccess) return e;
     const int copies = (size_t)32 * (nbins + 1) * sizeof(unsigned) <= 96 * 1024 ? 32 : 1;
     const size_t smem = sizeof(unsigned) * (size_t)copies * (nbins + 1);
-    // FP32 estimate error in bins: rounding of lo and of a - lo (each within
-    // one ulp of max(|lo|, |hi|)) times the scale, plus the scale's rounding
-    const double m = std::fmax(std::fabs(lo), std::fabs(hi));
-    const double ulp = m > 0.0 ? std::ldexp(1.0, std::ilogb(m) - 23) : 0.0;
-    const double err = 2.0 * ulp * (double)nbins / (hi - lo) + 4.0 * 6e-8 * (double)nbins;   // bins
-    const int fast = err <= 0.02 ? 1 : 0;
+    const double err = estimate_error(lo, hi, nbins);
+    const int fast = err <= kFastError ? 1 : 0;
     const float band = (float)std::fmax(4.0 * err, 1e-3);       // decide again this close to an edge
     float flo_in = (float)lo, fhi_in = (float)hi;
     if ((double)flo_in < lo) flo_in = std::nextafterf(flo_in, INFINITY);
     if ((double)fhi_in > hi) fhi_in = std::nextafterf(fhi_in, -INFINITY);
     float *edge = nullptr;
-    if (scratch && fast && (long long)v.nx * v.ny * v.nz >= kEdgesMinVoxels) {
+    if (scratch && histogram_wants_edges((long long)v.nx * v.ny * v.nz, lo, hi, nbins)) {
         edge = reinterpret_cast<float *>(static_cast<unsigned char *>(scratch) + kEdgeOffset);
         bin_edges_kernel<<<(unsigned)((nbins + kEdgeThreads - 1) / kEdgeThreads), kEdgeThreads, 0, s>>>(lo, hi, flo_in,
                                                                                                fhi_in, nbins, edge);

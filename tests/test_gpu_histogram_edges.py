@@ -41,3 +41,23 @@ def test_edges_near_zero(cube, lo, hi, nb):
     v = v[(v >= lo) & (v <= hi)]
     b = np.clip(np.floor((v - lo) / (hi - lo) * nb), 0, nb - 1).astype(np.int64)
     assert np.array_equal(got, np.bincount(b, minlength=nb))
+
+
+def test_no_scratch_where_the_edges_are_not_used():
+    """A small volume's histogram makes no device allocation: the failure armed
+    before it is left to the next call that makes one."""
+    torch = cuda_or_skip()
+    import paper_1211_4896_gb300 as P
+    from paper_1211_4896_gb300 import _lib as L
+    c = torch.randn((30, 40, 50), device="cuda")
+    vol = P.Volume(c, "f32")
+    try:
+        L.vr_debug_fail_alloc(0)
+        got = P.histogram(vol, -1.0, 1.0, 10)
+        with pytest.raises(L.VRError) as e:
+            P.moments(vol)
+        assert e.value.status == L.VR_ERR_OOM
+        assert int(got.sum()) == int((c.abs() <= 1.0).sum())
+    finally:
+        L.vr_debug_fail_alloc(-1)
+        vol.close()
