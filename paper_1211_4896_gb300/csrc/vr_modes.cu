@@ -161,10 +161,12 @@ __device__ __forceinline__ void mini_axis(float p, float rinv, int m, int &i0, f
 // sample are kept in registers (each x edge as its first value and its
 // difference): a ray stays in a mini-map cell for about a region's length,
 // and the march is bound by instructions, of which the eight loads and their
-// addresses were a fifth.
-struct SigmaMap {
+// addresses were a fifth.  I: the type that holds the map's point numbers,
+// long long from 2^31 points (regions of a voxel or two of a very large cube;
+// in every kernel it cost 0.7 to 4%).
+template <typename I> struct SigmaMap {
     MiniDev m;
-    mutable int at = -1;                           // the kept cell's first point
+    mutable I at = -1;                             // the kept cell's first point
     mutable float2 a[4], d[4];                     // edges (y0, z0), (y1, z0), (y0, z1), (y1, z1)
     __device__ __forceinline__ explicit SigmaMap(const MiniDev &md) : m(md) {}
     __device__ __forceinline__ float operator()(float v, const Cell &c) const
@@ -174,10 +176,11 @@ struct SigmaMap {
         mini_axis((float)c.x0 + c.fx, m.rx, m.mx, x0, wx);
         mini_axis((float)c.y0 + c.fy, m.ry, m.my, y0, wy);
         mini_axis((float)c.z0 + c.fz, m.rz, m.mz, z0, wz);
-        const int p = (z0 * m.my + y0) * m.mx + x0;     // fewer than 2^31 points
+        const I p = ((I)z0 * m.my + y0) * m.mx + x0;
         if (p != at) {
             at = p;
-            const int dx = m.mx > 1 ? 1 : 0, dy = m.my > 1 ? m.mx : 0, dz = m.mz > 1 ? m.mx * m.my : 0;
+            const int dx = m.mx > 1 ? 1 : 0, dy = m.my > 1 ? m.mx : 0;
+            const I dz = m.mz > 1 ? (I)m.mx * m.my : 0;
             if constexpr (kBoundsCheck) {
                 const long long n = (long long)m.mx * m.my * m.mz;
                 if (!index_ok(m.status, p, n) || !index_ok(m.status, (long long)p + dx + dy + dz, n)) {
@@ -209,14 +212,14 @@ struct SigmaMap {
 // and 1.07 at four (before: 1.02 ms at three eight-warp CTAs).
 constexpr int kSigmaThreads = 128;
 
-template <typename T, int LOG2B, int L, bool GROUPS>
+template <typename T, int LOG2B, int L, bool GROUPS, typename I>
 __global__ void __launch_bounds__(kSigmaThreads, 6) sigma_kernel(VolDev v, CamDev c, ParamDev p, MiniDev m, float4 *out,
                                                               uint32_t *nsamples, unsigned *counter, int tiles_x,
                                                               unsigned ntiles)
 {
     const int lane = threadIdx.x & 31;
-    const SigmaMap map(m);
-    const float z = GROUPS || skips_transparent<T, SigmaMap>() ? transparent_below(p) : 0.0f;
+    const SigmaMap<I> map(m);
+    const float z = GROUPS || skips_transparent<T, SigmaMap<I>>() ? transparent_below(p) : 0.0f;
     for (;;) {
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
@@ -229,8 +232,8 @@ __global__ void __launch_bounds__(kSigmaThreads, 6) sigma_kernel(VolDev v, CamDe
         const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
         int used;
-        if constexpr (GROUPS) used = march_group<T, LOG2B, L, kGroup, SigmaMap>(v, p, ray, hit, acc, z, map);
-        else used = march_ray<T, LOG2B, L, SigmaMap>(v, p, ray, hit, acc, z, map);
+        if constexpr (GROUPS) used = march_group<T, LOG2B, L, kGroup, SigmaMap<I>>(v, p, ray, hit, acc, z, map);
+        else used = march_ray<T, LOG2B, L, SigmaMap<I>>(v, p, ray, hit, acc, z, map);
         if (inside && !(GROUPS && lane >= 32 / kGroup)) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
     }
 }
@@ -268,6 +271,8 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
     m.ry = (float)(1.0 / region[1]);
     m.rz = (float)(1.0 / region[2]);
     m.status = v.status;
+    const bool wide = (long long)m.mx * m.my * m.mz > 0x7fffffffLL;
+    if (wide) groups = false;                      // built with a ray to a lane only
     int tiles_x;
     const unsigned ntiles = mode_tiles(c, groups, tiles_x);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
@@ -276,8 +281,9 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
-            auto fn = groups ? sigma_kernel<typename Y::type, Y::log2b, Y::order, true>
-                             : sigma_kernel<typename Y::type, Y::log2b, Y::order, false>;
+            auto fn = wide   ? sigma_kernel<typename Y::type, Y::log2b, Y::order, false, long long>
+                    : groups ? sigma_kernel<typename Y::type, Y::log2b, Y::order, true, int>
+                             : sigma_kernel<typename Y::type, Y::log2b, Y::order, false, int>;
             fn<<<persistent_grid(fn, ntiles, kSigmaThreads), kSigmaThreads, 0, s>>>(v, c, p, m, out, nsamples, counter, tiles_x,
                                                                     ntiles);
             return cudaGetLastError();
