@@ -404,9 +404,13 @@ bool sparse_view(const vr_volume *vol, const vr_camera *cam)
 
 // Whether a view is marched with several lanes to a ray: its rays share no
 // sectors, or it covers fewer than eight tiles of 32 rays an SM (the figures
-// stand at fwd_group_kernel).
+// stand at fwd_group_kernel).  VR_GROUPS=0 or 1 (read at each call) has every
+// view marched with a ray to a lane, or in groups: the same images, so that
+// tests reach both marches at any size.
 static bool march_in_groups(const vr_volume *vol, const vr_camera *cam)
 {
+    const char *e = std::getenv("VR_GROUPS");
+    if (e && (e[0] == '0' || e[0] == '1')) return e[0] == '1';
     return sparse_view(vol, cam) || covered_pixels(vol, cam) < 8.0 * 32.0 * (double)sm_count();
 }
 

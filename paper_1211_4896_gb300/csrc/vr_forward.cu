@@ -212,10 +212,13 @@ template <typename T, int LOG2B, int L>
 static FwdLaunch plan_fwd_t(const VolDev &v, const CamDev &c, bool groups)
 {
     FwdLaunch f;
+    if constexpr (is_blocked<T>::value) groups = true;      // only sparse views read these, and they march in groups
     const int tw = groups ? 2 : 8, th = groups ? 2 : 4;
     f.tiles_x = (c.W + tw - 1) / tw;
     f.ntiles = (unsigned)f.tiles_x * (unsigned)((c.H + th - 1) / th);
-    f.fn = groups ? fwd_group_kernel<T, LOG2B, L> : fwd_kernel<T, LOG2B, L>;
+    f.fn = fwd_group_kernel<T, LOG2B, L>;
+    if constexpr (!is_blocked<T>::value)
+        if (!groups) f.fn = fwd_kernel<T, LOG2B, L>;
     const int per_sm = groups ? occupancy_blocks((const void *)f.fn, kFwdThreads, 0)
                               : fwd_ctas_per_sm((const void *)f.fn, FwdCtaCap<T>::value);
     f.grid = fwd_grid(per_sm, f.ntiles);
