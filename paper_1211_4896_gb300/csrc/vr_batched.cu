@@ -156,7 +156,7 @@ struct BatchPlan {
     JobDev *djobs = nullptr;
     unsigned *counter = nullptr;       // one work counter per group, or (nodes) per job
     std::vector<JobDev> nodes;         // the jobs of a graph of single-view kernels, most expensive first
-    std::vector<bool> sparse;          // sparse_view of each
+    std::vector<Tiles> tiles;          // of each: sparse views march in groups
     int njobs = 0;
     Segment seg[kGroups];
     int log2_tw = 3;
@@ -335,7 +335,7 @@ static cudaError_t build_graph(BatchPlan *plan)
     e = cudaGraphAddMemsetNode(&reset, graph, nullptr, 0, &mp);
     for (size_t q = 0; q < plan->nodes.size() && e == cudaSuccess; ++q) {
         const JobDev &J = plan->nodes[q];
-        e = add_forward_node(graph, reset, J.v, plan->vols[0]->store_dtype, J.c, J.p, plan->sparse[q], J.out, J.nsamples,
+        e = add_forward_node(graph, reset, J.v, plan->vols[0]->store_dtype, J.c, J.p, plan->tiles[q], J.out, J.nsamples,
                              plan->counter + q);
     }
     for (int g = 0; g < kGroups && e == cudaSuccess && plan->nodes.empty(); ++g) {
@@ -473,7 +473,9 @@ extern "C" vr_status vr_render_batched(const vr_job *jobs, int n, const vr_batch
                              [&](int a, int b) { return cost[order[a]] > cost[order[b]]; });
             for (int q : by_cost) {
                 plan->nodes.push_back(hj[q]);
-                plan->sparse.push_back(sparse_view(jobs[order[q]].vol, &jobs[order[q]].cam));
+                const vr_job &J = jobs[order[q]];
+                plan->tiles.push_back(view_tiles(J.vol, &J.cam, sparse_view(J.vol, &J.cam) ? kInGroups : kRayPerLane, J.vol->origin,
+                                                 J.vol->dims));
             }
         }
         cudaError_t e = dev_alloc(reinterpret_cast<void **>(&plan->djobs), sizeof(JobDev) * (size_t)n);

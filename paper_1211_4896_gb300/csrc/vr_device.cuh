@@ -722,6 +722,11 @@ struct IdentityMap {
     __device__ __forceinline__ float operator()(float v, const Cell &) const { return v; }
 };
 
+// The same, for a march that looks every sample up: the batched kernel, whose
+// registers are full (a job's leading run kept in one more made 16 dense
+// 16-bit views with opaque tables 1% slower).
+struct LookAllUp : IdentityMap {};
+
 // Where a sample of the ray lies in the volume marched: at its position on the
 // ray, or, for a volume that holds part of a larger grid, that position less
 // the part's offset (exact for 0 <= off <= p).
@@ -735,11 +740,6 @@ struct PartOfGrid {
         return make_float3(p.x - off.x, p.y - off.y, p.z - off.z);
     }
 };
-
-// The same, for a march that looks every sample up: the batched kernel, whose
-// registers are full (a job's leading run kept in one more made 16 dense
-// 16-bit views with opaque tables 1% slower).
-struct LookAllUp : IdentityMap {};
 
 // Whether a march leaves out the table lookup and the composite of samples
 // below z (transparent_below): the two 16-byte table loads of a sample are a
@@ -897,14 +897,38 @@ __device__ __forceinline__ int march_group(const VolDev &v, const ParamDev &p, c
     return used;
 }
 
-// Lanes to a ray of the kernels that march in groups, and the pixel of a
-// lane's ray in their 2 x 2 tiles.
+// Lanes to a ray of the kernels that march in groups.
 constexpr int kGroup = 8;
 
-__device__ __forceinline__ int2 group_pixel(unsigned tile, int tiles_x)
+// A lane's pixel: whether its ray is marched and whether the lane writes it.
+struct LanePixel {
+    int i, j;
+    bool march, writes;
+};
+
+template <bool GROUPS> __device__ __forceinline__ LanePixel lane_pixel(const Tiles &t, unsigned tile, int W, int H)
 {
-    const int r = threadIdx.x & (32 / kGroup - 1);
-    return make_int2((int)(tile % tiles_x) * 2 + (r & 1), (int)(tile / tiles_x) * 2 + (r >> 1));
+    const int lane = threadIdx.x & 31;
+    LanePixel q;
+    if constexpr (!GROUPS) {
+        const int2 at = tile_pixel(lane, 3);
+        q.i = (int)(tile % t.tiles_x) * 8 + at.x;
+        q.j = (int)(tile / t.tiles_x) * 4 + at.y;
+        q.march = q.writes = q.i < W && q.j < H;
+    } else if (tile < t.nmarch) {
+        const int r = lane & (32 / kGroup - 1);
+        q.i = t.x0 + (int)(tile % t.tiles_x) * 2 + (r & 1);
+        q.j = t.y0 + (int)(tile / t.tiles_x) * 2 + (r >> 1);
+        q.march = q.i < W && q.j < H;
+        q.writes = q.march && lane < 32 / kGroup;
+    } else {
+        const unsigned b = tile - t.nmarch;
+        q.i = (int)(b % t.blocks_x) * 8 + (lane & 7);
+        q.j = (int)(b / t.blocks_x) * 4 + (lane >> 3);
+        q.march = false;
+        q.writes = q.i < W && q.j < H && !((unsigned)(q.i - t.x0) < (unsigned)t.w && (unsigned)(q.j - t.y0) < (unsigned)t.h);
+    }
+    return q;
 }
 
 __device__ __forceinline__ void write_pixel(const ParamDev &p, const Composite &acc, int used, float4 *out,

@@ -40,8 +40,7 @@ template <> struct FwdDepth<TexLayers<float>> { static constexpr int value = 2; 
 
 template <typename T, int LOG2B, int L>
 __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
-                                                           uint32_t *nsamples, unsigned *counter, int tiles_x,
-                                                           unsigned ntiles)
+                                                           uint32_t *nsamples, unsigned *counter, Tiles t)
 {
     const int lane = threadIdx.x & 31;
     const float z = skips_transparent<T, IdentityMap>() ? transparent_below(p) : 0.0f;
@@ -49,16 +48,13 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
-        if (tile >= ntiles) break;
-        const int2 at = tile_pixel(lane, 3);
-        const int i = (int)(tile % tiles_x) * 8 + at.x;
-        const int j = (int)(tile / tiles_x) * 4 + at.y;
-        const bool inside = i < c.W && j < c.H;
+        if (tile >= t.ntiles) break;
+        const LanePixel px = lane_pixel<false>(t, tile, c.W, c.H);
         Ray ray;
-        const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
+        const bool hit = px.march && setup_ray(c, v.nx, v.ny, v.nz, p.step, px.i, px.j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
         const int used = march_ray<T, LOG2B, L, IdentityMap, FwdDepth<T>::value>(v, p, ray, hit, acc, z);
-        if (inside) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
+        if (px.writes) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)px.j * c.W + px.i);
     }
 }
 
@@ -85,8 +81,7 @@ __global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kerne
 // view of a 128^3 cube, all of it covered, 82 -> 87.
 template <typename T, int LOG2B, int L>
 __global__ void __launch_bounds__(kFwdThreads, 3 * kPerSm) fwd_group_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
-                                                                uint32_t *nsamples, unsigned *counter, int tiles_x,
-                                                                unsigned ntiles)
+                                                                uint32_t *nsamples, unsigned *counter, Tiles t)
 {
     const int lane = threadIdx.x & 31;
     const float z = transparent_below(p);
@@ -94,15 +89,13 @@ __global__ void __launch_bounds__(kFwdThreads, 3 * kPerSm) fwd_group_kernel(VolD
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
-        if (tile >= ntiles) break;
-        const int2 at = group_pixel(tile, tiles_x);
-        const int i = at.x, j = at.y;
-        const bool inside = i < c.W && j < c.H;
+        if (tile >= t.ntiles) break;
+        const LanePixel px = lane_pixel<true>(t, tile, c.W, c.H);
         Ray ray;
-        const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
+        const bool hit = px.march && setup_ray(c, v.nx, v.ny, v.nz, p.step, px.i, px.j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
         const int used = march_group<T, LOG2B, L, kGroup>(v, p, ray, hit, acc, z);
-        if (inside && lane < 32 / kGroup) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
+        if (px.writes) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)px.j * c.W + px.i);
     }
 }
 
@@ -203,61 +196,59 @@ static unsigned fwd_grid(int per_sm, unsigned tiles)
 
 // A view's kernel and its grid.
 struct FwdLaunch {
-    void (*fn)(VolDev, CamDev, ParamDev, float4 *, uint32_t *, unsigned *, int, unsigned) = nullptr;
-    int tiles_x = 0;
-    unsigned ntiles = 0, grid = 0;
+    void (*fn)(VolDev, CamDev, ParamDev, float4 *, uint32_t *, unsigned *, Tiles) = nullptr;
+    unsigned grid = 0;
 };
 
 template <typename T, int LOG2B, int L>
-static FwdLaunch plan_fwd_t(const VolDev &v, const CamDev &c, bool groups)
+static FwdLaunch plan_fwd_t(const VolDev &v, const CamDev &c, const Tiles &t)
 {
     FwdLaunch f;
-    if constexpr (is_blocked<T>::value) groups = true;      // only sparse views read these, and they march in groups
-    const int tw = groups ? 2 : 8, th = groups ? 2 : 4;
-    f.tiles_x = (c.W + tw - 1) / tw;
-    f.ntiles = (unsigned)f.tiles_x * (unsigned)((c.H + th - 1) / th);
     f.fn = fwd_group_kernel<T, LOG2B, L>;
-    if constexpr (!is_blocked<T>::value)
-        if (!groups) f.fn = fwd_kernel<T, LOG2B, L>;
-    const int per_sm = groups ? occupancy_blocks((const void *)f.fn, kFwdThreads, 0)
-                              : fwd_ctas_per_sm((const void *)f.fn, FwdCtaCap<T>::value);
-    f.grid = fwd_grid(per_sm, f.ntiles);
-    log_line("forward %dx%d: layout order %d%s, %u tiles of %dx%d rays, %d lane(s) to a ray, grid %u x %d threads (%d per SM)",
-             c.W, c.H, v.order, layout_name(v), f.ntiles, tw, th, groups ? kGroup : 1, f.grid, kFwdThreads, per_sm);
+    if constexpr (is_blocked<T>::value) {      // only sparse views read these, and they march in groups
+        if (!t.groups) return FwdLaunch();
+    } else {
+        if (!t.groups) f.fn = fwd_kernel<T, LOG2B, L>;
+    }
+    const int per_sm = t.groups ? occupancy_blocks((const void *)f.fn, kFwdThreads, 0)
+                                : fwd_ctas_per_sm((const void *)f.fn, FwdCtaCap<T>::value);
+    f.grid = fwd_grid(per_sm, t.ntiles);
+    log_line("forward %dx%d: layout order %d%s, %u tiles of %s rays, %d lane(s) to a ray, grid %u x %d threads (%d per SM)",
+             c.W, c.H, v.order, layout_name(v), t.nmarch, t.groups ? "2x2" : "8x4", t.groups ? kGroup : 1, f.grid,
+             kFwdThreads, per_sm);
     return f;
 }
 
-static FwdLaunch plan_fwd(const VolDev &v, vr_dtype dt, const CamDev &c, bool groups)
+static FwdLaunch plan_fwd(const VolDev &v, vr_dtype dt, const CamDev &c, const Tiles &t)
 {
     return visit_layout_all(
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
-            return plan_fwd_t<typename Y::type, Y::log2b, Y::order>(v, c, groups);
+            return plan_fwd_t<typename Y::type, Y::log2b, Y::order>(v, c, t);
         },
         FwdLaunch());
 }
 
-// groups: eight lanes to a ray (march_in_groups).
-cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
+cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s)
 {
-    const FwdLaunch f = plan_fwd(v, dt, c, groups);
+    const FwdLaunch f = plan_fwd(v, dt, c, t);
     if (!f.fn) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
-    f.fn<<<f.grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, f.tiles_x, f.ntiles);
+    f.fn<<<f.grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, t);
     return cudaGetLastError();
 }
 
 // The same view as a kernel node after `reset`, which clears its counter.
 cudaError_t add_forward_node(cudaGraph_t graph, cudaGraphNode_t reset, const VolDev &v, vr_dtype dt, const CamDev &c,
-                             const ParamDev &p, bool groups, float4 *out, uint32_t *nsamples, unsigned *counter)
+                             const ParamDev &p, const Tiles &t, float4 *out, uint32_t *nsamples, unsigned *counter)
 {
-    FwdLaunch f = plan_fwd(v, dt, c, groups);
+    const FwdLaunch f = plan_fwd(v, dt, c, t);
     if (!f.fn) return cudaErrorInvalidValue;
     void *args[] = {const_cast<VolDev *>(&v), const_cast<CamDev *>(&c), const_cast<ParamDev *>(&p), &out, &nsamples,
-                    &counter, &f.tiles_x, &f.ntiles};
+                    &counter, const_cast<Tiles *>(&t)};
     cudaKernelNodeParams kp = {};
     kp.func = (void *)f.fn;
     kp.gridDim = dim3(f.grid);

@@ -58,6 +58,19 @@ struct VolDev {
     unsigned *status;      // the volume's status word (timeouts, caught out-of-range indices)
 };
 
+// How a view's pixels are handed out: 8 x 4 tiles with a ray to a lane, or
+// (groups) with eight lanes to a ray, 2 x 2 tiles over the pixels [x0, x0 + w) x
+// [y0, y0 + h) around the volume, then 8 x 4 blocks over the whole image for
+// the pixels outside of them, whose rays miss it.
+struct Tiles {
+    bool groups = false;
+    int tiles_x = 0;           // tiles across
+    unsigned nmarch = 0;       // tiles marched
+    unsigned ntiles = 0;       // with the blocks
+    int blocks_x = 0;          // blocks across
+    int x0 = 0, y0 = 0, w = 0, h = 0;
+};
+
 // Dense copy of the volume, x fastest, rows padded to a multiple of 8
 // elements so that 16-byte asynchronous copies of any x-aligned run are legal.
 struct DenseDev {
@@ -145,10 +158,10 @@ int sm_count();
 cudaError_t launch_brick(const void *src, vr_dtype src_dtype, vr_volume *vol, cudaStream_t s);
 cudaError_t launch_rebrick(const vr_volume *src, vr_volume *dst, cudaStream_t s);   // same dims and storage
 vr_status build_texture(vr_volume *vol, cudaStream_t s);
-cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
+cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s);
 cudaError_t add_forward_node(cudaGraph_t graph, cudaGraphNode_t reset, const VolDev &v, vr_dtype dt, const CamDev &c,
-                             const ParamDev &p, bool groups, float4 *out, uint32_t *nsamples, unsigned *counter);
+                             const ParamDev &p, const Tiles &t, float4 *out, uint32_t *nsamples, unsigned *counter);
 bool sparse_view(const vr_volume *vol, const vr_camera *cam);     // rays too far apart to share sectors
 cudaError_t launch_forward_texture(const vr_volume *vol, const CamDev &c, const ParamDev &p, float4 *out,
                                    uint32_t *nsamples, unsigned *counter, cudaStream_t s);
@@ -163,6 +176,10 @@ inline bool copy_paired(int copy) { return copy >= 3 && copy < 6; }
 inline bool copy_blocked(int copy) { return copy >= 6 && copy < 9; }
 inline bool copy_layers(int copy) { return copy >= 9 && copy < 12; }
 inline int copy_order(int copy) { return copy >= 9 ? copy - 9 : (copy >= 6 ? copy - 6 : (copy >= 3 ? copy - 3 : copy)); }
+// Which march a view takes: as asked, or by the pixels it covers.
+enum March { kRayPerLane, kInGroups, kAuto };
+Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const double grid_origin[3],
+                 const int64_t grid_dims[3]);
 // Whether copy id `copy` exists on vol.
 bool copy_built(const vr_volume *vol, int copy);
 // Elements per brick of a blocked copy (B = 1 << log2b; elem_bytes 4 or 2).
@@ -210,17 +227,17 @@ int occupancy_blocks(const void *fn, int threads, size_t smem);
 cudaError_t launch_wait_selftest(unsigned *status, cudaStream_t s);
 cudaError_t launch_bounds_selftest(unsigned *status, cudaStream_t s);
 // Other uses of the march (vr_modes.cu).
-cudaError_t launch_mip(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
+cudaError_t launch_mip(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t, float4 *out,
                        uint32_t *nsamples, unsigned *counter, cudaStream_t s);
-cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups,
+cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t,
                          const float *minimap,
                          const int region[3], float4 *out, uint32_t *nsamples, unsigned *counter, cudaStream_t s);
 cudaError_t launch_minimap(const VolDev &v, vr_dtype dt, const int region[3], float *dev_out, cudaStream_t s);
 cudaError_t launch_profile(const VolDev &v, vr_dtype dt, const CamDev &c, float step, int i, int j, float *values,
                            unsigned max_values, unsigned *count, cudaStream_t s);
-// Sort-last sub-box render and depth-ordered composite (vr_modes.cu).
+// Sort-last sub-box render and depth-ordered composite (vr_sortlast.cu).
 constexpr int kMaxPartials = 64;
-cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, const int lo[3],
+cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t, const int lo[3],
                           const int hi[3], const int gdim[3], const int off[3], float4 *partial, float *depth,
                           uint32_t *count, unsigned *counter, cudaStream_t s);
 cudaError_t launch_composite(int k, const float *const *partials, const float *const *depths, long long npx,

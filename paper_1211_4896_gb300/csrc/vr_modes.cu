@@ -68,8 +68,6 @@ __device__ __forceinline__ float march_max(const VolDev &v, const ParamDev &p, c
     return m;
 }
 
-// The pixel is the table entry of the largest value composited once over
-// the background; a ray that misses the box shows the background.
 // The same maximum with eight lanes to a ray (as march_group): each lane its
 // own samples, then the group's largest, on every lane of the group.
 template <typename T, int LOG2B, int L>
@@ -100,27 +98,26 @@ __device__ __forceinline__ float march_max_group(const VolDev &v, const ParamDev
     return m;
 }
 
+// The pixel is the table entry of the largest value composited once over
+// the background; a ray that misses the box shows the background.
 template <typename T, int LOG2B, int L, bool GROUPS>
 __global__ void __launch_bounds__(kModeThreads, ModeMinBlocks<T>::value) mip_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
-                                                            uint32_t *nsamples, unsigned *counter, int tiles_x,
-                                                            unsigned ntiles)
+                                                            uint32_t *nsamples, unsigned *counter, Tiles t)
 {
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
-        if (tile >= ntiles) break;
-        const int2 at = mode_pixel<GROUPS>(tile, tiles_x);
-        const int i = at.x, j = at.y;
-        const bool inside = i < c.W && j < c.H;
+        if (tile >= t.ntiles) break;
+        const LanePixel px = lane_pixel<GROUPS>(t, tile, c.W, c.H);
         Ray ray;
-        const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
+        const bool hit = px.march && setup_ray(c, v.nx, v.ny, v.nz, p.step, px.i, px.j, ray);
         float m;
         if constexpr (GROUPS) m = march_max_group<T, LOG2B, L>(v, p, ray, hit);
         else m = march_max<T, LOG2B, L, ModeDepth<T>::value>(v, p, ray, hit);
-        if (!inside || (GROUPS && lane >= 32 / kGroup)) continue;
-        const long long px = (long long)j * c.W + i;
+        if (!px.writes) continue;
+        const long long at = (long long)px.j * c.W + px.i;
         float4 o = p.bg;
         if (hit) {
             TfPos tp;
@@ -129,8 +126,8 @@ __global__ void __launch_bounds__(kModeThreads, ModeMinBlocks<T>::value) mip_ker
             o = make_float4(fmaf(a, e.x, t * p.bg.x), fmaf(a, e.y, t * p.bg.y), fmaf(a, e.z, t * p.bg.z),
                             fmaf(t, p.bg.w, a));
         }
-        out[px] = o;
-        if (nsamples) nsamples[px] = hit ? (uint32_t)ray.n : 0u;
+        out[at] = o;
+        if (nsamples) nsamples[at] = hit ? (uint32_t)ray.n : 0u;
     }
 }
 
@@ -214,8 +211,7 @@ constexpr int kSigmaThreads = 128;
 
 template <typename T, int LOG2B, int L, bool GROUPS, typename I>
 __global__ void __launch_bounds__(kSigmaThreads, 6) sigma_kernel(VolDev v, CamDev c, ParamDev p, MiniDev m, float4 *out,
-                                                              uint32_t *nsamples, unsigned *counter, int tiles_x,
-                                                              unsigned ntiles)
+                                                              uint32_t *nsamples, unsigned *counter, Tiles t)
 {
     const int lane = threadIdx.x & 31;
     const SigmaMap<I> map(m);
@@ -224,41 +220,36 @@ __global__ void __launch_bounds__(kSigmaThreads, 6) sigma_kernel(VolDev v, CamDe
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
-        if (tile >= ntiles) break;
-        const int2 at = mode_pixel<GROUPS>(tile, tiles_x);
-        const int i = at.x, j = at.y;
-        const bool inside = i < c.W && j < c.H;
+        if (tile >= t.ntiles) break;
+        const LanePixel px = lane_pixel<GROUPS>(t, tile, c.W, c.H);
         Ray ray;
-        const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
+        const bool hit = px.march && setup_ray(c, v.nx, v.ny, v.nz, p.step, px.i, px.j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
         int used;
         if constexpr (GROUPS) used = march_group<T, LOG2B, L, kGroup, SigmaMap<I>>(v, p, ray, hit, acc, z, map);
         else used = march_ray<T, LOG2B, L, SigmaMap<I>>(v, p, ray, hit, acc, z, map);
-        if (inside && !(GROUPS && lane >= 32 / kGroup)) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)j * c.W + i);
+        if (px.writes) write_pixel(p, acc, hit ? used : 0, out, nsamples, (long long)px.j * c.W + px.i);
     }
 }
 
-cudaError_t launch_mip(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, float4 *out,
+cudaError_t launch_mip(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t, float4 *out,
                        uint32_t *nsamples, unsigned *counter, cudaStream_t s)
 {
-    int tiles_x;
-    const unsigned ntiles = mode_tiles(c, groups, tiles_x);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     return visit_layout_tex(
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
-            auto fn = groups ? mip_kernel<typename Y::type, Y::log2b, Y::order, true>
+            auto fn = t.groups ? mip_kernel<typename Y::type, Y::log2b, Y::order, true>
                              : mip_kernel<typename Y::type, Y::log2b, Y::order, false>;
-            fn<<<persistent_grid(fn, ntiles), kModeThreads, 0, s>>>(v, c, p, out, nsamples, counter, tiles_x,
-                                                                    ntiles);
+            fn<<<persistent_grid(fn, t.ntiles), kModeThreads, 0, s>>>(v, c, p, out, nsamples, counter, t);
             return cudaGetLastError();
         },
         cudaErrorInvalidValue);
 }
 
-cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups,
+cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t,
                          const float *minimap,
                          const int region[3], float4 *out, uint32_t *nsamples, unsigned *counter, cudaStream_t s)
 {
@@ -272,20 +263,17 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
     m.rz = (float)(1.0 / region[2]);
     m.status = v.status;
     const bool wide = (long long)m.mx * m.my * m.mz > 0x7fffffffLL;
-    if (wide) groups = false;                      // built with a ray to a lane only
-    int tiles_x;
-    const unsigned ntiles = mode_tiles(c, groups, tiles_x);
+    if (wide && t.groups) return cudaErrorInvalidValue;           // built with a ray to a lane only
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     return visit_layout_tex(
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
-            auto fn = wide   ? sigma_kernel<typename Y::type, Y::log2b, Y::order, false, long long>
-                    : groups ? sigma_kernel<typename Y::type, Y::log2b, Y::order, true, int>
-                             : sigma_kernel<typename Y::type, Y::log2b, Y::order, false, int>;
-            fn<<<persistent_grid(fn, ntiles, kSigmaThreads), kSigmaThreads, 0, s>>>(v, c, p, m, out, nsamples, counter, tiles_x,
-                                                                    ntiles);
+            auto fn = wide     ? sigma_kernel<typename Y::type, Y::log2b, Y::order, false, long long>
+                    : t.groups ? sigma_kernel<typename Y::type, Y::log2b, Y::order, true, int>
+                               : sigma_kernel<typename Y::type, Y::log2b, Y::order, false, int>;
+            fn<<<persistent_grid(fn, t.ntiles, kSigmaThreads), kSigmaThreads, 0, s>>>(v, c, p, m, out, nsamples, counter, t);
             return cudaGetLastError();
         },
         cudaErrorInvalidValue);

@@ -8,24 +8,10 @@ namespace vr {
 
 constexpr int kModeThreads = 256;
 
-// Pixel of a lane's ray: its warp's 8 x 4 tile, or (GROUPS) 2 x 2 tile with
-// eight lanes to a ray.  These kernels march in groups for the views that
-// vr_render does (march_in_groups): 150 x 100 views of a 200 x 220 x 190 float
-// cube, maximum 207 -> 35 us, sigma clipping with its mini-map 378 -> 88, six
-// sub-boxes and their composite 842 -> 240 (bound by the host's calls).
-template <bool GROUPS> __device__ __forceinline__ int2 mode_pixel(unsigned tile, int tiles_x)
-{
-    if (GROUPS) return group_pixel(tile, tiles_x);
-    const int2 at = tile_pixel(threadIdx.x & 31, 3);
-    return make_int2((int)(tile % tiles_x) * 8 + at.x, (int)(tile / tiles_x) * 4 + at.y);
-}
-
-// Tiles of an image, across and in all.
-inline unsigned mode_tiles(const CamDev &c, bool groups, int &tiles_x)
-{
-    tiles_x = groups ? (c.W + 1) / 2 : (c.W + 7) / 8;
-    return (unsigned)tiles_x * (unsigned)(groups ? (c.H + 1) / 2 : (c.H + 3) / 4);
-}
+// These kernels march in groups for the views that vr_render does: 150 x 100
+// views of a 200 x 220 x 190 float cube, maximum 207 -> 35 us, sigma clipping
+// with its mini-map 378 -> 88, six sub-boxes and their composite 842 -> 240
+// (bound by the host's calls).
 
 // Persistent grid of a kernel over its tiles.
 template <typename K>

@@ -95,7 +95,7 @@ struct SubBox {
 template <typename T, int LOG2B, int L, bool GROUPS>
 __global__ void __launch_bounds__(kModeThreads, SubMinBlocks<T>::value) subbox_kernel(
     VolDev v, CamDev c, ParamDev p, int3 lo, int3 hi, SubBox box, int3 gdim, float3 off, float4 *partial, float *depth,
-    uint32_t *count, unsigned *counter, int tiles_x, unsigned ntiles)
+    uint32_t *count, unsigned *counter, Tiles t)
 {
     const int lane = threadIdx.x & 31;
     const float z = GROUPS || skips_transparent<T, IdentityMap>() ? transparent_below(p) : 0.0f;
@@ -103,14 +103,12 @@ __global__ void __launch_bounds__(kModeThreads, SubMinBlocks<T>::value) subbox_k
         unsigned tile = 0;
         if (lane == 0) tile = atomicAdd(counter, 1u);
         tile = __shfl_sync(kFull, tile, 0);
-        if (tile >= ntiles) break;
-        const int2 at = mode_pixel<GROUPS>(tile, tiles_x);
-        const int i = at.x, j = at.y;
-        const bool inside_img = i < c.W && j < c.H;
+        if (tile >= t.ntiles) break;
+        const LanePixel px = lane_pixel<GROUPS>(t, tile, c.W, c.H);
         Ray ray;
         // rays and samples of the whole grid (gdim voxels; the camera is in its
         // coordinates); the volume holds its voxels from off on
-        bool active = inside_img && setup_ray(c, gdim.x, gdim.y, gdim.z, p.step, i, j, ray);
+        bool active = px.march && setup_ray(c, gdim.x, gdim.y, gdim.z, p.step, px.i, px.j, ray);
         int2 run = make_int2(0, 0);
         if (active) {
             // a ray that misses the sub-box widened by one voxel has no sample in it
@@ -129,20 +127,18 @@ __global__ void __launch_bounds__(kModeThreads, SubMinBlocks<T>::value) subbox_k
         else
             march_ray<T, LOG2B, L, IdentityMap, SubDepth<T>::value, PartOfGrid>(v, p, ray, active, acc, z, IdentityMap(),
                                                                                 PartOfGrid{off}, run.x);
-        if (!inside_img || (GROUPS && lane >= 32 / kGroup)) continue;
-        const long long px = (long long)j * c.W + i;
-        partial[px] = make_float4(acc.r, acc.g, acc.b, acc.T);
-        depth[px] = active ? fmaf((float)run.x + 0.5f, p.step, ray.s_in) - eye_param(c, i, j) : INFINITY;
-        if (count) count[px] = (uint32_t)(run.y - run.x);
+        if (!px.writes) continue;
+        const long long at = (long long)px.j * c.W + px.i;
+        partial[at] = make_float4(acc.r, acc.g, acc.b, acc.T);
+        depth[at] = active ? fmaf((float)run.x + 0.5f, p.step, ray.s_in) - eye_param(c, px.i, px.j) : INFINITY;
+        if (count) count[at] = (uint32_t)(run.y - run.x);
     }
 }
 
-cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, bool groups, const int lo[3],
+cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t, const int lo[3],
                           const int hi[3], const int gdim[3], const int off[3], float4 *partial, float *depth,
                           uint32_t *count, unsigned *counter, cudaStream_t s)
 {
-    int tiles_x;
-    const unsigned ntiles = mode_tiles(c, groups, tiles_x);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     const int3 l3 = make_int3(lo[0], lo[1], lo[2]), h3 = make_int3(hi[0], hi[1], hi[2]);
@@ -160,10 +156,10 @@ cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const P
         v, dt,
         [&](auto lay) {
             using Y = decltype(lay);
-            auto fn = groups ? subbox_kernel<typename Y::type, Y::log2b, Y::order, true>
+            auto fn = t.groups ? subbox_kernel<typename Y::type, Y::log2b, Y::order, true>
                              : subbox_kernel<typename Y::type, Y::log2b, Y::order, false>;
-            fn<<<persistent_grid(fn, ntiles), kModeThreads, 0, s>>>(v, c, q, l3, h3, box, g3, o3, partial, depth, count,
-                                                                    counter, tiles_x, ntiles);
+            fn<<<persistent_grid(fn, t.ntiles), kModeThreads, 0, s>>>(v, c, q, l3, h3, box, g3, o3, partial, depth, count,
+                                                                      counter, t);
             return cudaGetLastError();
         },
         cudaErrorInvalidValue);
