@@ -768,17 +768,17 @@ __device__ __forceinline__ void march_step(const VolDev &v, const ParamDev &p, c
         fetch_corners<T, LOG2B, L>(v, nxt, fn);
     }
     const float val = map(interp_corners(cur, fc), cur);
+    if (!(skips_transparent<T, Map>() && fmaf(val, p.su, p.ou) < z)) {
+        TfPos tp;
+        const float4 e = tf_lookup_l1(p, val, tp);
+        const float aT = e.w * acc.T;
+        acc.r = fmaf(aT, e.x, acc.r);
+        acc.g = fmaf(aT, e.y, acc.g);
+        acc.b = fmaf(aT, e.z, acc.b);
+        acc.T = fmaf(-e.w, acc.T, acc.T);
+    }
     ++k;
-    if (!more) active = false;
-    if (skips_transparent<T, Map>() && fmaf(val, p.su, p.ou) < z) return;
-    TfPos tp;
-    const float4 e = tf_lookup_l1(p, val, tp);
-    const float aT = e.w * acc.T;
-    acc.r = fmaf(aT, e.x, acc.r);
-    acc.g = fmaf(aT, e.y, acc.g);
-    acc.b = fmaf(aT, e.z, acc.b);
-    acc.T = fmaf(-e.w, acc.T, acc.T);
-    if (acc.T <= p.t_stop) active = false;
+    if (!more || acc.T <= p.t_stop) active = false;
 }
 
 // The loop body is unrolled over depth + 1 register sets that take turns, so

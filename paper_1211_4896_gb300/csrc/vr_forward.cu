@@ -22,8 +22,12 @@ namespace vr {
 // Two-warp CTAs: warps do not depend on one another, and small CTAs hand an
 // SM's slots on warp pair by warp pair at the end of a view (views that follow
 // each other in a batch's graph: 16 uneven cubes 2.04 -> 1.89 ms against
-// eight-warp CTAs).
+// eight-warp CTAs).  Eight-warp CTAs for the paired copies, whose dense views
+// are not graph nodes of their own as a rule: neighbouring tiles then share an
+// SM's L1 (16-bit views with an opaque table 1 to 4% faster).
 constexpr int kFwdThreads = 64;
+template <typename T> struct FwdThreads { static constexpr int value = kFwdThreads; };
+template <typename S> struct FwdThreads<Pair<S>> { static constexpr int value = 256; };
 constexpr int kPerSm = 256 / kFwdThreads;            // CTAs that make eight warps
 
 // Resident warps the register budget is sized for, and samples whose gathers
@@ -34,12 +38,12 @@ constexpr int kPerSm = 256 / kFwdThreads;            // CTAs that make eight war
 // copies; 24 for the other brick layouts, with the march's own depth.
 template <typename T> struct FwdMinBlocks { static constexpr int value = 3 * kPerSm; };
 template <> struct FwdMinBlocks<TexLayers<float>> { static constexpr int value = 4 * kPerSm; };
-template <typename S> struct FwdMinBlocks<Pair<S>> { static constexpr int value = 4 * kPerSm; };
+template <typename S> struct FwdMinBlocks<Pair<S>> { static constexpr int value = 4; };
 template <typename T> struct FwdDepth { static constexpr int value = Pipeline<T>::depth; };
 template <> struct FwdDepth<TexLayers<float>> { static constexpr int value = 2; };
 
 template <typename T, int LOG2B, int L>
-__global__ void __launch_bounds__(kFwdThreads, FwdMinBlocks<T>::value) fwd_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
+__global__ void __launch_bounds__(FwdThreads<T>::value, FwdMinBlocks<T>::value) fwd_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
                                                            uint32_t *nsamples, unsigned *counter, Tiles t)
 {
     const int lane = threadIdx.x & 31;
@@ -162,14 +166,14 @@ int occupancy_blocks(const void *fn, int threads, size_t smem)
 // Resident CTAs per SM for the persistent forward grid: the occupancy limit,
 // at most `cap` (0: none), or eight warps for each VR_FWD_CTAS_PER_SM when set
 // (a tuning knob: fewer resident warps thrash the L1 and L2 less).
-static int fwd_ctas_per_sm(const void *fn, int cap)
+static int fwd_ctas_per_sm(const void *fn, int threads, int cap)
 {
-    const int occ = occupancy_blocks(fn, kFwdThreads, 0);
+    const int occ = occupancy_blocks(fn, threads, 0);
     static const int env = [] {
         const char *s = std::getenv("VR_FWD_CTAS_PER_SM");
         return s ? std::atoi(s) : 0;
     }();
-    const int want = env > 0 ? env * kPerSm : cap;
+    const int want = env > 0 ? env * (256 / threads) : cap;
     return (want > 0 && want < occ) ? want : occ;
 }
 
@@ -188,9 +192,9 @@ static const char *layout_name(const VolDev &v)
 
 // Persistent grid of `tiles` tiles: per_sm CTAs on each SM, no more than
 // there are tiles for.
-static unsigned fwd_grid(int per_sm, unsigned tiles)
+static unsigned fwd_grid(int per_sm, int threads, unsigned tiles)
 {
-    const unsigned grid = (unsigned)(per_sm * sm_count()), useful = (tiles + kFwdThreads / 32 - 1) / (kFwdThreads / 32);
+    const unsigned warps = (unsigned)threads / 32, grid = (unsigned)(per_sm * sm_count()), useful = (tiles + warps - 1) / warps;
     return grid < useful ? grid : (useful ? useful : 1u);
 }
 
@@ -198,6 +202,7 @@ static unsigned fwd_grid(int per_sm, unsigned tiles)
 struct FwdLaunch {
     void (*fn)(VolDev, CamDev, ParamDev, float4 *, uint32_t *, unsigned *, Tiles) = nullptr;
     unsigned grid = 0;
+    int threads = kFwdThreads;
 };
 
 template <typename T, int LOG2B, int L>
@@ -208,14 +213,14 @@ static FwdLaunch plan_fwd_t(const VolDev &v, const CamDev &c, const Tiles &t)
     if constexpr (is_blocked<T>::value) {      // only sparse views read these, and they march in groups
         if (!t.groups) return FwdLaunch();
     } else {
-        if (!t.groups) f.fn = fwd_kernel<T, LOG2B, L>;
+        if (!t.groups) f.fn = fwd_kernel<T, LOG2B, L>, f.threads = FwdThreads<T>::value;
     }
-    const int per_sm = t.groups ? occupancy_blocks((const void *)f.fn, kFwdThreads, 0)
-                                : fwd_ctas_per_sm((const void *)f.fn, FwdCtaCap<T>::value);
-    f.grid = fwd_grid(per_sm, t.ntiles);
+    const int per_sm = t.groups ? occupancy_blocks((const void *)f.fn, f.threads, 0)
+                                : fwd_ctas_per_sm((const void *)f.fn, f.threads, FwdCtaCap<T>::value);
+    f.grid = fwd_grid(per_sm, f.threads, t.ntiles);
     log_line("forward %dx%d: layout order %d%s, %u tiles of %s rays, %d lane(s) to a ray, grid %u x %d threads (%d per SM)",
              c.W, c.H, v.order, layout_name(v), t.nmarch, t.groups ? "2x2" : "8x4", t.groups ? kGroup : 1, f.grid,
-             kFwdThreads, per_sm);
+             f.threads, per_sm);
     return f;
 }
 
@@ -237,7 +242,7 @@ cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const 
     if (!f.fn) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
-    f.fn<<<f.grid, kFwdThreads, 0, s>>>(v, c, p, out, nsamples, counter, t);
+    f.fn<<<f.grid, f.threads, 0, s>>>(v, c, p, out, nsamples, counter, t);
     return cudaGetLastError();
 }
 
@@ -252,7 +257,7 @@ cudaError_t add_forward_node(cudaGraph_t graph, cudaGraphNode_t reset, const Vol
     cudaKernelNodeParams kp = {};
     kp.func = (void *)f.fn;
     kp.gridDim = dim3(f.grid);
-    kp.blockDim = dim3(kFwdThreads);
+    kp.blockDim = dim3(f.threads);
     kp.kernelParams = args;
     cudaGraphNode_t node = nullptr;
     return cudaGraphAddKernelNode(&node, graph, &reset, 1, &kp);
@@ -264,7 +269,7 @@ cudaError_t launch_forward_texture(const vr_volume *vol, const CamDev &c, const 
     const int tiles_x = (c.W + 7) / 8, tiles_y = (c.H + 3) / 4;
     const unsigned ntiles = (unsigned)tiles_x * (unsigned)tiles_y;
     const int per_sm = occupancy_blocks((const void *)fwd_tex_kernel, kFwdThreads, 0);
-    const unsigned grid = fwd_grid(per_sm, ntiles);
+    const unsigned grid = fwd_grid(per_sm, kFwdThreads, ntiles);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     fwd_tex_kernel<<<grid, kFwdThreads, 0, s>>>(vol->tex, (int)vol->dims[0], (int)vol->dims[1], (int)vol->dims[2],
