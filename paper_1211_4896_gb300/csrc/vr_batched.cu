@@ -65,6 +65,8 @@ __global__ void __launch_bounds__(kBatThreads, LOG2_WPT ? 0 : BatMinBlocks<T>::v
     const int lane = threadIdx.x & 31;
     const int tw = 1 << log2_tw;
     const int2 at = tile_pixel(lane, log2_tw);
+    int last_job = -1;                       // the job z belongs to
+    float z = 0.0f;
     for (;;) {
         unsigned tile = 0;
         if constexpr (LOG2_WPT == 0) {
@@ -93,11 +95,15 @@ __global__ void __launch_bounds__(kBatThreads, LOG2_WPT ? 0 : BatMinBlocks<T>::v
         const CamDev c = J.c;
         const ParamDev p = J.p;
         const VolDev v = J.v;
+        if (skips_transparent<T, IdentityMap>() && lo != last_job) {
+            last_job = lo;
+            z = transparent_below(p);
+        }
         const bool inside = i < c.W && j < c.H;
         Ray ray;
         const bool hit = inside && setup_ray(c, v.nx, v.ny, v.nz, p.step, i, j, ray);
         Composite acc{0.0f, 0.0f, 0.0f, 1.0f};
-        const int used = march_ray<T, LOG2B, L, LookAllUp>(v, p, ray, hit, acc, 0.0f);
+        const int used = march_ray<T, LOG2B, L>(v, p, ray, hit, acc, z);
         if (inside) write_pixel(p, acc, hit ? used : 0, J.out, J.nsamples, (long long)j * c.W + i);
     }
 }

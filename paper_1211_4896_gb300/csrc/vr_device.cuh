@@ -722,11 +722,6 @@ struct IdentityMap {
     __device__ __forceinline__ float operator()(float v, const Cell &) const { return v; }
 };
 
-// The same, for a march that looks every sample up: the batched kernel, whose
-// registers are full (a job's leading run kept in one more made 16 dense
-// 16-bit views with opaque tables 1% slower).
-struct LookAllUp : IdentityMap {};
-
 // Where a sample of the ray lies in the volume marched: at its position on the
 // ray, or, for a volume that holds part of a larger grid, that position less
 // the part's offset (exact for 0 <= off <= p).
@@ -743,13 +738,15 @@ struct PartOfGrid {
 
 // Whether a march leaves out the table lookup and the composite of samples
 // below z (transparent_below): the two 16-byte table loads of a sample are a
-// third of the L1 wavefronts of a brick layout's march (16-bit view of a
-// 705 x 611 x 833 cube 758 -> 694 us), and sigma clipping is bound by
-// instructions (1% faster).  The plain march through texture layers waits on
-// the texture unit's return path either way, and the branch costs it 1-4%.
+// third of the L1 wavefronts of a brick layout's march, and sigma clipping is
+// bound by instructions (1% faster).  16-bit views against a march that looks
+// every sample up, the benchmark's ramp: 9 to 20% faster, with an opaque table
+// from 4% faster to 5% slower; batches of them (five lists, both 16-bit types)
+// 14 to 22% and 0 to 4% faster.  The plain march through texture layers waits
+// on the texture unit's return path either way, and the branch costs it 1-4%.
 template <typename T, typename Map> __device__ constexpr bool skips_transparent()
 {
-    return !std::is_same<Map, LookAllUp>::value && (!is_layers<T>::value || !std::is_same<Map, IdentityMap>::value);
+    return !is_layers<T>::value || !std::is_same<Map, IdentityMap>::value;
 }
 
 // One sample: composites (cur, fc) and, while the ray goes on, issues the
