@@ -415,13 +415,14 @@ bool sparse_view(const vr_volume *vol, const vr_camera *cam)
 }
 
 // Whether a view is marched with several lanes to a ray: its rays share no
-// sectors, or it covers fewer than eight tiles of 32 rays an SM (the figures
-// stand at fwd_group_kernel).  VR_GROUPS=0 or 1 (read at each call) has every
-// view marched with a ray to a lane, or in groups: the same images, so that
-// tests reach both marches at any size.  rect: NULL when any pixel may see the
-// volume.
-static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const CornerRect *rect)
+// sectors, or it covers few pixels, fewer than 256 an SM (from 80 an SM on only
+// with a table that suits: by_table); the figures stand at fwd_group_kernel.
+// VR_GROUPS=0 or 1 (read at each call) has every view marched with a ray to a
+// lane, or in groups: the same images, so that tests reach both marches at any
+// size.  rect: NULL when any pixel may see the volume.
+static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const CornerRect *rect, bool &by_table)
 {
+    by_table = false;
     const char *e = std::getenv("VR_GROUPS");
     if (e && (e[0] == '0' || e[0] == '1')) return e[0] == '1';
     double covered = (double)cam->width * cam->height;
@@ -430,7 +431,9 @@ static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const Co
         for (int a = 0; a < 2; ++a)
             covered *= std::fmax(std::fmin(rect->hi[a], a ? cam->height : cam->width) - std::fmax(rect->lo[a], 0.0), 0.0);
     }
-    return covered < 8.0 * 32.0 * (double)sm_count() || sparse_view(vol, cam);
+    const double sms = (double)sm_count();
+    if (covered < 80.0 * sms || sparse_view(vol, cam)) return true;
+    return by_table = covered < 256.0 * sms;
 }
 
 // The tiles of a view.  In groups only the pixels around the volume are handed
@@ -448,7 +451,11 @@ Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const 
     CornerRect q, g;
     const bool seen = march != kRayPerLane && corner_rect(vol->origin, vol->spacing, vol->dims, cam, q);
     Tiles t;
-    t.groups = march == kInGroups || (march == kAuto && march_in_groups(vol, cam, seen ? &q : nullptr));
+    t.groups = march == kInGroups;
+    if (march == kByPixels || march == kByTable) {
+        t.groups = march_in_groups(vol, cam, seen ? &q : nullptr, t.by_table);
+        t.by_table = t.by_table && march == kByTable;
+    }
     if (!t.groups) {
         t.tiles_x = (W + 7) / 8;
         t.nmarch = t.ntiles = (unsigned)t.tiles_x * (unsigned)((H + 3) / 4);
@@ -468,17 +475,16 @@ Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const 
     t.h = (t.h + 1) & ~1;
     t.tiles_x = t.w / 2;
     t.nmarch = t.ntiles = (unsigned)t.tiles_x * (unsigned)(t.h / 2);
-    if (t.w < W || t.h < H) {
-        t.blocks_x = (W + 7) / 8;
-        t.ntiles += (unsigned)t.blocks_x * (unsigned)((H + 3) / 4);
-    }
+    t.blocks_x = (W + 7) / 8;
+    t.nblocks = (unsigned)t.blocks_x * (unsigned)((H + 3) / 4);
+    if (t.w < W || t.h < H) t.ntiles += t.nblocks;
     return t;
 }
 
 // (blocked copies, which only sparse views read, are marched in groups alone)
 static Tiles tiles_of(const vr_volume *vol, const vr_camera *cam, int copy)
 {
-    return view_tiles(vol, cam, copy_blocked(copy) ? kInGroups : kAuto, vol->origin, vol->dims);
+    return view_tiles(vol, cam, copy_blocked(copy) ? kInGroups : kByTable, vol->origin, vol->dims);
 }
 
 // Brick copy for a camera.  Its fastest axis is the one along which the
@@ -996,7 +1002,9 @@ vr_status vr_render(vr_volume_t vol, const vr_camera *cam, const vr_params *para
                                 reinterpret_cast<float4 *>(dev_rgba_out), dev_nsamples_out, ctr, s);
     } else if (params->mode == VR_MODE_MIP) {
         const int copy = preferred_copy(vol, cam, true, s, kReadsLayers);
-        e = launch_mip(vol_dev_copy(vol, copy), vol->store_dtype, c, p, tiles_of(vol, cam, copy),
+        // (the maximum composites nothing: the larger limit whatever the table)
+        e = launch_mip(vol_dev_copy(vol, copy), vol->store_dtype, c, p,
+                       view_tiles(vol, cam, kByPixels, vol->origin, vol->dims),
                        reinterpret_cast<float4 *>(dev_rgba_out), dev_nsamples_out, ctr, s);
     } else if (params->mode == VR_MODE_SIGMA) {
         const int copy = preferred_copy(vol, cam, true, s, kReadsLayers);
@@ -1215,7 +1223,7 @@ static vr_status subbox_of(vr_volume_t vol, const int64_t gdims[3], const int64_
     const int off[3] = {(int)offset[0], (int)offset[1], (int)offset[2]};
     const int copy = preferred_copy(vol, cam, true, s, kReadsLayers);
     cudaError_t e = launch_subbox(vol_dev_copy(vol, copy), vol->store_dtype, c, p,
-                                  view_tiles(vol, cam, kAuto, gorigin, gdims), cell_lo, cell_hi, gd, off, reinterpret_cast<float4 *>(dev_partial), dev_depth,
+                                  view_tiles(vol, cam, kByTable, gorigin, gdims), cell_lo, cell_hi, gd, off, reinterpret_cast<float4 *>(dev_partial), dev_depth,
                                   dev_count, ctr, s);
     if (e != cudaSuccess) return cuda_fail(e, who);
     return VR_OK;

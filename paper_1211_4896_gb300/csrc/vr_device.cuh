@@ -897,6 +897,13 @@ __device__ __forceinline__ int march_group(const VolDev &v, const ParamDev &p, c
 // Lanes to a ray of the kernels that march in groups.
 constexpr int kGroup = 8;
 
+// Whether a view launched both ways (Tiles::by_table) is marched by the other
+// kernel.  Called by whole warps.
+template <bool GROUPS> __device__ __forceinline__ bool not_this_march(const Tiles &t, const ParamDev &p)
+{
+    return t.by_table && (transparent_below(p) == -INFINITY) == GROUPS;
+}
+
 // A lane's pixel: whether its ray is marched and whether the lane writes it.
 struct LanePixel {
     int i, j;

@@ -46,6 +46,7 @@ template <typename T, int LOG2B, int L>
 __global__ void __launch_bounds__(FwdThreads<T>::value, FwdMinBlocks<T>::value) fwd_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
                                                            uint32_t *nsamples, unsigned *counter, Tiles t)
 {
+    if (not_this_march<false>(t, p)) return;
     const int lane = threadIdx.x & 31;
     const float z = skips_transparent<T, IdentityMap>() ? transparent_below(p) : 0.0f;
     for (;;) {
@@ -76,17 +77,24 @@ __global__ void __launch_bounds__(FwdThreads<T>::value, FwdMinBlocks<T>::value) 
 // where rays are long and transparent and lose 15% where they end after 50
 // samples; two rounds of gathers in flight are the same trade.
 //
-// Views whose volume covers few pixels (fewer than eight 8 x 4 tiles an SM):
-// with a ray to each lane they leave the SMs a few warps each, which wait out
-// every gather's latency along the whole ray.  128 x 120 x 140 cube, 320 x 200
-// pixels: float 94 -> 40 us, opaque table 83 -> 57, float16 87 -> 40.  With
-// more tiles the composite's shuffles cost more than the latency: 400 x 320
-// pixels 105 -> 60, but with the opaque table 94 -> 104; a face-on 256 x 256
-// view of a 128^3 cube, all of it covered, 82 -> 87.
+// Views whose volume covers few pixels: with a ray to each lane they leave the
+// SMs a few warps each, which wait out every gather's latency along the whole
+// ray.  Against a ray to a lane (five cubes from 60^3 to 400 x 300 x 350, three
+// directions, float and float16, step 0.7; slowest to fastest), by covered
+// pixels: 2500: 1.8 to 3.4 times as fast with the benchmark's ramp, 1.5 to 1.9
+// with an opaque table; 10 000: 1.8 to 3.0 and 1.2 to 1.7; 16 000: 1.6 to 3.8 and
+// 0.9 to 1.8; 24 000: 1.3 to 3.5 and 0.75 to 1.6; 38 000: 1.2 to 3.8 and 0.6 to
+// 1.5: an opaque table's samples are all composited, and their shuffles cost
+// more than the latency once an SM has a few tiles.  So views of up to 80
+// covered pixels an SM march in groups, and up to 256 an SM those whose table
+// begins with transparent entries.  Only the device has read the table, so
+// these are launched both ways (Tiles::by_table; both marches in one kernel
+// cost each of them 10% to a factor of 4).
 template <typename T, int LOG2B, int L>
 __global__ void __launch_bounds__(kFwdThreads, 3 * kPerSm) fwd_group_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
                                                                 uint32_t *nsamples, unsigned *counter, Tiles t)
 {
+    if (not_this_march<true>(t, p)) return;
     const int lane = threadIdx.x & 31;
     const float z = transparent_below(p);
     for (;;) {
@@ -238,12 +246,16 @@ static FwdLaunch plan_fwd(const VolDev &v, vr_dtype dt, const CamDev &c, const T
 cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const ParamDev &p, const Tiles &t, float4 *out,
                            uint32_t *nsamples, unsigned *counter, cudaStream_t s)
 {
-    const FwdLaunch f = plan_fwd(v, dt, c, t);
-    if (!f.fn) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    f.fn<<<f.grid, f.threads, 0, s>>>(v, c, p, out, nsamples, counter, t);
-    return cudaGetLastError();
+    auto launch = [&](const Tiles &q) {
+        const FwdLaunch f = plan_fwd(v, dt, c, q);
+        if (!f.fn) return cudaErrorInvalidValue;
+        f.fn<<<f.grid, f.threads, 0, s>>>(v, c, p, out, nsamples, counter, q);
+        return cudaGetLastError();
+    };
+    if (e == cudaSuccess) e = launch(t);
+    if (e == cudaSuccess && t.by_table) e = launch(lane_tiles(t));    // one of the two returns at once
+    return e;
 }
 
 // The same view as a kernel node after `reset`, which clears its counter.

@@ -61,15 +61,29 @@ struct VolDev {
 // How a view's pixels are handed out: 8 x 4 tiles with a ray to a lane, or
 // (groups) with eight lanes to a ray, 2 x 2 tiles over the pixels [x0, x0 + w) x
 // [y0, y0 + h) around the volume, then 8 x 4 blocks over the whole image for
-// the pixels outside of them, whose rays miss it.
+// the pixels outside of them, whose rays miss it.  by_table: a view that is
+// better off in groups when its table begins with transparent entries and with
+// a ray to a lane when it does not is launched both ways, and the kernel that
+// the table does not suit returns at once (not_this_march).
 struct Tiles {
-    bool groups = false;
+    bool groups = false, by_table = false;
     int tiles_x = 0;           // tiles across
     unsigned nmarch = 0;       // tiles marched
     unsigned ntiles = 0;       // with the blocks
     int blocks_x = 0;          // blocks across
+    unsigned nblocks = 0;
     int x0 = 0, y0 = 0, w = 0, h = 0;
 };
+
+// The tiles with which the same view marches with a ray to a lane.
+inline Tiles lane_tiles(const Tiles &t)
+{
+    Tiles q;
+    q.by_table = t.by_table;
+    q.tiles_x = t.blocks_x;
+    q.nmarch = q.ntiles = t.nblocks;
+    return q;
+}
 
 // Dense copy of the volume, x fastest, rows padded to a multiple of 8
 // elements so that 16-byte asynchronous copies of any x-aligned run are legal.
@@ -176,8 +190,9 @@ inline bool copy_paired(int copy) { return copy >= 3 && copy < 6; }
 inline bool copy_blocked(int copy) { return copy >= 6 && copy < 9; }
 inline bool copy_layers(int copy) { return copy >= 9 && copy < 12; }
 inline int copy_order(int copy) { return copy >= 9 ? copy - 9 : (copy >= 6 ? copy - 6 : (copy >= 3 ? copy - 3 : copy)); }
-// Which march a view takes: as asked, or by the pixels it covers.
-enum March { kRayPerLane, kInGroups, kAuto };
+// Which march a view takes: as asked, or by the pixels it covers (kByPixels) and,
+// between two limits, its table (kByTable).
+enum March { kRayPerLane, kInGroups, kByPixels, kByTable };
 Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const double grid_origin[3],
                  const int64_t grid_dims[3]);
 // Whether copy id `copy` exists on vol.

@@ -213,6 +213,7 @@ template <typename T, int LOG2B, int L, bool GROUPS, typename I>
 __global__ void __launch_bounds__(kSigmaThreads, 6) sigma_kernel(VolDev v, CamDev c, ParamDev p, MiniDev m, float4 *out,
                                                               uint32_t *nsamples, unsigned *counter, Tiles t)
 {
+    if (not_this_march<GROUPS>(t, p)) return;
     const int lane = threadIdx.x & 31;
     const SigmaMap<I> map(m);
     const float z = GROUPS || skips_transparent<T, SigmaMap<I>>() ? transparent_below(p) : 0.0f;
@@ -274,6 +275,11 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
                     : t.groups ? sigma_kernel<typename Y::type, Y::log2b, Y::order, true, int>
                                : sigma_kernel<typename Y::type, Y::log2b, Y::order, false, int>;
             fn<<<persistent_grid(fn, t.ntiles, kSigmaThreads), kSigmaThreads, 0, s>>>(v, c, p, m, out, nsamples, counter, t);
+            if (t.by_table) {                     // both ways: one of the two returns at once
+                const Tiles q = lane_tiles(t);
+                fn = sigma_kernel<typename Y::type, Y::log2b, Y::order, false, int>;
+                fn<<<persistent_grid(fn, q.ntiles, kSigmaThreads), kSigmaThreads, 0, s>>>(v, c, p, m, out, nsamples, counter, q);
+            }
             return cudaGetLastError();
         },
         cudaErrorInvalidValue);

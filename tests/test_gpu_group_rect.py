@@ -109,3 +109,35 @@ def test_sparse_views_of_a_batch(torch, monkeypatch, store):
             assert torch.equal(a, j["out"]) and torch.equal(na, j["nsamples"])
     finally:
         vol.close()
+
+
+@pytest.mark.parametrize("store", ["f32", "f16"])
+@pytest.mark.parametrize("size", [100, 111, 150, 190, 205])       # 80 and 256 covered pixels an SM of 152 lie between them
+def test_the_march_that_the_table_picks(torch, monkeypatch, store, size):
+    """Views between the two limits, whose kernel marches in groups or with a
+    ray to a lane by the table: no leading zero opacities, one (not enough to
+    leave out a sample), two, most."""
+    import paper_1211_4896_gb300 as P
+    vol = P.Volume(synth.hi_cube(DIMS, n_blobs=5, n_disks=0, seed=2).cuda(), store)
+    mm = P.minimap(vol, (5, 6, 7))
+    cams = [synth.camera_ortho((10.0, 16.5, -60.0), (0, 0, 1), (0, 1, 0), 18.0, size, size - 1),
+            synth.camera_persp((80.0, -50.0, 90.0), (-0.62, 0.6, -0.7), (0, 1, 0), 12.0, size + 3, size)]
+    try:
+        for run in (0, 1, 2, 200):
+            tab = synth.tf_random_pwl(seed=3, K=256, alpha_max=0.4)
+            tab[:, 3] += 0.01
+            tab[:run, 3] = 0.0
+            tf = torch.from_numpy(tab).cuda()
+            for cam in cams:
+                calls = [lambda: P.render(vol, cam, tf, -3.0, 30.0, 0.4, 0.97),
+                         lambda: P.render(vol, cam, tf, -3.0, 30.0, 0.4, mode=P.VR_MODE_MIP),
+                         lambda: P.render(vol, cam, tf, 0.0, 8.0, 0.4, 0.97, mode=P.VR_MODE_SIGMA, minimap=mm, region=(5, 6, 7)),
+                         lambda: P.render_subbox(vol, cam, tf, -3.0, 30.0, 0.4, (3, 5, 7), (18, 30, 20))]
+                for call in calls:
+                    monkeypatch.setenv("VR_GROUPS", "0")
+                    a = call()
+                    monkeypatch.delenv("VR_GROUPS")
+                    for x, y in zip(a, call()):
+                        assert torch.equal(x, y)
+    finally:
+        vol.close()
