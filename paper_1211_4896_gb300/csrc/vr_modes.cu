@@ -299,23 +299,22 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
 // subtraction, product and addition carried along (Knuth's two-sum and the
 // fused product error): about 25 FP32 operations a voxel.  The low parts are
 // plain FP32 sums, so the two are brought back to hi + lo with |lo| below half
-// an ulp of hi every kRenorm values: each addition's error then stays below
-// 2^-25 kRenorm / 2 ulps of hi, and that of the sums of the 2^13 values that a
-// thread has at most below 2^-30 of them, if all errors pointed one way.  The
-// variance S2 / n - (S1 / n)^2 is formed in FP64 and loses what the shift is
-// away from the mean: where (S1 / n)^2 exceeds 16 variances (a first voxel four
-// deviations off: 6e-5 of the regions of noise), a second pass has the mean
-// found as its shift, and so do deviations whose squares leave the float
-// range, scaled by a power of two.  Against 64 bits, restated on the CPU over
-// noise, outliers up to 1e7 as the first voxel and quantised data in up to
-// 128^3: 1e-12 of the deviation at most (without the second pass 2.6e-6),
-// where rounding the result to float is 6e-8.
+// an ulp of hi after kRenorm values or a column of them.  The variance
+// S2 / n - (S1 / n)^2 is formed in FP64 and loses what the shift is away from the
+// mean: where (S1 / n)^2 exceeds 256 variances (a first voxel 16 deviations off,
+// hardly ever but in outliers) a second pass has the mean found as its shift,
+// and so do deviations whose squares leave the float range, scaled by a power of
+// two.  Against 64 bits, restated on the CPU over noise, outliers up to 1e7 as
+// the first voxel and quantised data in regions of up to 128^3: 2e-9 of the
+// deviation at most (5e-8 with no renorm, 4e-6 without the second pass), where
+// rounding the result to float is 6e-8.
 // A region with a voxel that is not finite needs no sums; one above 2^21
 // voxels, or whose differences overflow, takes two FP64 passes.
 // ---------------------------------------------------------------------------
 
-constexpr int kMiniThreads = 256;                  // 64 or 128 for regions of few voxels
+constexpr int kMiniThreads = 256;                  // 64 or 128 for regions of few voxels (region_sums: at most 8 warps)
 constexpr long long kMiniMaxOnePass = 1LL << 21;
+constexpr float kMiniMinFar = 1e-12f, kMiniMaxFar = 1e18f;        // largest deviations whose squares need no scale
 
 __device__ __forceinline__ double block_sum(double x, double *red)
 {
@@ -350,7 +349,7 @@ __device__ __forceinline__ float brick_voxel(const VolDev &v, int x, int y, int 
 }
 
 // A sum kept as hi + lo, hi the rounded sum so far.
-constexpr int kRenorm = 32;
+constexpr int kRenorm = 128;
 struct TwoFloat {
     float hi = 0.0f, lo = 0.0f;
     __device__ __forceinline__ void add(float x)
@@ -366,6 +365,15 @@ struct TwoFloat {
         add(x);
     }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    // the sum over the warp, on every lane
+    __device__ __forceinline__ void warp_sum()
+    {
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h = __shfl_xor_sync(kFull, hi, o), l = __shfl_xor_sync(kFull, lo, o);
+            add(h);
+            lo = __fadd_rn(lo, l);
+        }
+    }
 };
 
 // A region of voxels [x0, x0 + lx) x [y0, y0 + ly) x [z0, z0 + lz).
@@ -374,7 +382,7 @@ struct Region {
 };
 
 // Calls f(value) for every voxel of the region (each thread its own) and
-// after() after every U of a thread's.
+// after(n) after at most n of a thread's, those of one (x, y).
 template <typename T, typename F, typename G>
 __device__ __forceinline__ void for_region(const VolDev &v, const Region &q, F &&f, G &&after)
 {
@@ -401,8 +409,8 @@ __device__ __forceinline__ void for_region(const VolDev &v, const Region &q, F &
                     if (z + u * sz >= q.lz) break;
                     f(to_f(raw[u]));
                 }
-                after(U);
             }
+            after(q.lz / sz + 1);
         }
     }
 }
@@ -441,14 +449,31 @@ __device__ __forceinline__ RegionSums region_sums(const VolDev &v, const Region 
                 run = 0;
             }
         });
-    RegionSums r;
-    r.s1 = block_sum(s1.value(), red);
-    r.s2 = block_sum(s2.value(), red);
+    // over the warps in FP64 by the first of them (on every thread they would take
+    // a fifth of a 32^3 region's time)
+    s1.warp_sum();
+    s2.warp_sum();
     for (int o = 16; o > 0; o >>= 1) far = fmaxf(far, __shfl_xor_sync(kFull, far, o));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = (int)(blockDim.x >> 5);
+    double *far_of = red + 16;                    // red: 8 warps' s1, s2, far, and the three totals
+    __syncthreads();                              // red[] may still be read by the previous call
+    if (lane == 0) red[warp] = s1.value(), red[8 + warp] = s2.value(), far_of[warp] = (double)far;
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)far;
+    if (warp == 0) {
+        double x = lane < warps ? red[lane] : 0.0, y = lane < warps ? red[8 + lane] : 0.0;
+        far = lane < warps ? (float)far_of[lane] : 0.0f;
+        for (int o = 4; o > 0; o >>= 1) {
+            x += __shfl_xor_sync(kFull, x, o);
+            y += __shfl_xor_sync(kFull, y, o);
+            far = fmaxf(far, __shfl_xor_sync(kFull, far, o));
+        }
+        if (lane == 0) red[24] = x, red[25] = y, red[26] = (double)far;
+    }
     __syncthreads();
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) far = fmaxf(far, (float)red[w]);
+    RegionSums r;
+    r.s1 = red[24];
+    r.s2 = red[25];
+    far = (float)red[26];
     r.far = far;
     return r;
 }
@@ -473,23 +498,19 @@ __device__ double2 region_two_pass(const VolDev &v, const Region &q, double *red
     return make_double2(mean, block_sum(ss, red) / (double)cnt);
 }
 
-// The region's mean and variance by the one-pass sums.
+// What the first pass's sums t about `shift` do not settle (see above).  A call of
+// its own, so that its registers do not bound the first pass.
 template <typename T>
-__device__ double2 region_one_pass(const VolDev &v, const Region &q, double *red)
+__device__ __noinline__ double2 region_again(const VolDev &v, const Region &q, float shift, RegionSums t, double *red)
 {
     const double n = (double)((long long)q.lx * q.ly * q.lz);
-    float shift = brick_voxel<T>(v, q.x0, q.y0, q.z0);
-    RegionSums t = region_sums<T, false>(v, q, shift, 1.0f, red);
-    double m = t.s1 / n, var = t.s2 / n - m * m;
-    const bool in_range = t.far >= 1e-12f && t.far <= 1e18f;
     if (isfinite(t.s1)) {                                       // so every voxel is finite
-        if (t.far == 0.0f || (in_range && m * m <= 16.0 * var)) return make_double2((double)shift + m, fmax(var, 0.0));
-        shift = (float)((double)shift + m);
+        shift = (float)((double)shift + t.s1 / n);
+        const bool in_range = t.far >= kMiniMinFar && t.far <= kMiniMaxFar;
         const float scale = in_range ? 1.0f : ldexpf(1.0f, min(max(-ilogbf(t.far), -126), 126));
         t = region_sums<T, true>(v, q, shift, scale, red);
         if (isfinite(t.s1) && isfinite(t.s2)) {
-            m = t.s1 / n;
-            var = fmax(t.s2 / n - m * m, 0.0) / ((double)scale * (double)scale);
+            const double m = t.s1 / n, var = fmax(t.s2 / n - m * m, 0.0) / ((double)scale * (double)scale);
             return make_double2((double)shift + m / (double)scale, var);
         }
     } else {
@@ -501,6 +522,18 @@ __device__ double2 region_one_pass(const VolDev &v, const Region &q, double *red
         if (up || down) return make_double2(up && down ? (double)NAN : (up ? INFINITY : -INFINITY), (double)NAN);
     }
     return region_two_pass<T>(v, q, red);
+}
+
+// The region's mean and variance by the one-pass sums.
+template <typename T>
+__device__ __forceinline__ double2 region_one_pass(const VolDev &v, const Region &q, double *red)
+{
+    const float shift = brick_voxel<T>(v, q.x0, q.y0, q.z0);
+    const RegionSums t = region_sums<T, false>(v, q, shift, 1.0f, red);
+    const double n = (double)((long long)q.lx * q.ly * q.lz), m = t.s1 / n, var = t.s2 / n - m * m;
+    const bool settled = t.far == 0.0f || (t.far >= kMiniMinFar && t.far <= kMiniMaxFar && m * m <= 256.0 * var);
+    if (isfinite(t.s1) && settled) return make_double2((double)shift + m, fmax(var, 0.0));
+    return region_again<T>(v, q, shift, t, red);
 }
 
 template <typename T>
