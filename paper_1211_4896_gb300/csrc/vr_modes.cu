@@ -57,7 +57,11 @@ __device__ __forceinline__ float march_max(const VolDev &v, const ParamDev &p, c
     }
     while (__any_sync(kFull, active)) {
         if constexpr (D == 1) {
+            // a vote for each step: with one for two, 16-bit views (30 of 35 to
+            // 2000 MB of paired copies) ran at 0.88 to 1.06 of this speed, the
+            // largest the slowest
             if (active) step(c0, f0, c1, f1);
+            if (!__any_sync(kFull, active)) break;
             if (active) step(c1, f1, c0, f0);
         } else {
             if (active) step(c0, f0, c2, f2);
