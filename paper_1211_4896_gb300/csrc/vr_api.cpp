@@ -415,12 +415,13 @@ bool sparse_view(const vr_volume *vol, const vr_camera *cam)
 }
 
 // Whether a view is marched with several lanes to a ray: its rays share no
-// sectors, or it covers few pixels, fewer than 256 an SM (from 80 an SM on only
-// with a table that suits: by_table); the figures stand at fwd_group_kernel.
+// sectors, or it covers few pixels (kGroupPixels an SM; from any_table an SM on
+// only with a table that suits: by_table).
 // VR_GROUPS=0 or 1 (read at each call) has every view marched with a ray to a
 // lane, or in groups: the same images, so that tests reach both marches at any
 // size.  rect: NULL when any pixel may see the volume.
-static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const CornerRect *rect, bool &by_table)
+static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const CornerRect *rect, double any_table,
+                            bool &by_table)
 {
     by_table = false;
     const char *e = std::getenv("VR_GROUPS");
@@ -432,8 +433,8 @@ static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const Co
             covered *= std::fmax(std::fmin(rect->hi[a], a ? cam->height : cam->width) - std::fmax(rect->lo[a], 0.0), 0.0);
     }
     const double sms = (double)sm_count();
-    if (covered < 80.0 * sms || sparse_view(vol, cam)) return true;
-    return by_table = covered < 256.0 * sms;
+    if (covered < any_table * sms || sparse_view(vol, cam)) return true;
+    return by_table = covered < kGroupPixels * sms;
 }
 
 // The tiles of a view.  In groups only the pixels around the volume are handed
@@ -444,7 +445,7 @@ static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const Co
 // rays' 32-bit positions, which are relative to the grid the camera is set up
 // in (grid_origin and grid_dims: the volume's own, or the larger grid that it
 // is part of).
-Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const double grid_origin[3],
+Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, double any_table, const double grid_origin[3],
                  const int64_t grid_dims[3])
 {
     const int W = cam->width, H = cam->height;
@@ -452,10 +453,7 @@ Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const 
     const bool seen = march != kRayPerLane && corner_rect(vol->origin, vol->spacing, vol->dims, cam, q);
     Tiles t;
     t.groups = march == kInGroups;
-    if (march == kByPixels || march == kByTable) {
-        t.groups = march_in_groups(vol, cam, seen ? &q : nullptr, t.by_table);
-        t.by_table = t.by_table && march == kByTable;
-    }
+    if (march == kAuto) t.groups = march_in_groups(vol, cam, seen ? &q : nullptr, any_table, t.by_table);
     if (!t.groups) {
         t.tiles_x = (W + 7) / 8;
         t.nmarch = t.ntiles = (unsigned)t.tiles_x * (unsigned)((H + 3) / 4);
@@ -482,9 +480,9 @@ Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const 
 }
 
 // (blocked copies, which only sparse views read, are marched in groups alone)
-static Tiles tiles_of(const vr_volume *vol, const vr_camera *cam, int copy)
+static Tiles tiles_of(const vr_volume *vol, const vr_camera *cam, int copy, double any_table)
 {
-    return view_tiles(vol, cam, copy_blocked(copy) ? kInGroups : kByTable, vol->origin, vol->dims);
+    return view_tiles(vol, cam, copy_blocked(copy) ? kInGroups : kAuto, any_table, vol->origin, vol->dims);
 }
 
 // Brick copy for a camera.  Its fastest axis is the one along which the
@@ -1003,14 +1001,14 @@ vr_status vr_render(vr_volume_t vol, const vr_camera *cam, const vr_params *para
     } else if (params->mode == VR_MODE_MIP) {
         const int copy = preferred_copy(vol, cam, true, s, kReadsLayers);
         // (the maximum composites nothing: the larger limit whatever the table)
-        e = launch_mip(vol_dev_copy(vol, copy), vol->store_dtype, c, p,
-                       view_tiles(vol, cam, kByPixels, vol->origin, vol->dims),
+        e = launch_mip(vol_dev_copy(vol, copy), vol->store_dtype, c, p, tiles_of(vol, cam, copy, kGroupPixels),
                        reinterpret_cast<float4 *>(dev_rgba_out), dev_nsamples_out, ctr, s);
     } else if (params->mode == VR_MODE_SIGMA) {
         const int copy = preferred_copy(vol, cam, true, s, kReadsLayers);
         int64_t points = 1;                        // a map of 2^31 and more is read with a ray to a lane
         for (int a = 0; a < 3; ++a) points *= (vol->dims[a] + params->minimap_region[a] - 1) / params->minimap_region[a];
-        const Tiles t = points > INT32_MAX ? view_tiles(vol, cam, kRayPerLane, vol->origin, vol->dims) : tiles_of(vol, cam, copy);
+        const Tiles t = points > INT32_MAX ? view_tiles(vol, cam, kRayPerLane, 0.0, vol->origin, vol->dims)
+                                            : tiles_of(vol, cam, copy, kModePixels);
         e = launch_sigma(vol_dev_copy(vol, copy), vol->store_dtype, c, p, t, params->minimap, params->minimap_region,
                          reinterpret_cast<float4 *>(dev_rgba_out), dev_nsamples_out, ctr, s);
     } else if (params->filter == VR_FILTER_TEXTURE) {
@@ -1024,7 +1022,7 @@ vr_status vr_render(vr_volume_t vol, const vr_camera *cam, const vr_params *para
                                   dev_nsamples_out, ctr, status_word(vol), s);
     } else {
         const int copy = preferred_copy(vol, cam, true, s, kReadsBlocked | kReadsLayers);
-        e = launch_forward(vol_dev_copy(vol, copy), vol->store_dtype, c, p, tiles_of(vol, cam, copy),
+        e = launch_forward(vol_dev_copy(vol, copy), vol->store_dtype, c, p, tiles_of(vol, cam, copy, kCompositePixels),
                            reinterpret_cast<float4 *>(dev_rgba_out), dev_nsamples_out, ctr, s);
     }
     if (e != cudaSuccess) return cuda_fail(e, "vr_render launch");
@@ -1223,7 +1221,7 @@ static vr_status subbox_of(vr_volume_t vol, const int64_t gdims[3], const int64_
     const int off[3] = {(int)offset[0], (int)offset[1], (int)offset[2]};
     const int copy = preferred_copy(vol, cam, true, s, kReadsLayers);
     cudaError_t e = launch_subbox(vol_dev_copy(vol, copy), vol->store_dtype, c, p,
-                                  view_tiles(vol, cam, kByTable, gorigin, gdims), cell_lo, cell_hi, gd, off, reinterpret_cast<float4 *>(dev_partial), dev_depth,
+                                  view_tiles(vol, cam, kAuto, kModePixels, gorigin, gdims), cell_lo, cell_hi, gd, off, reinterpret_cast<float4 *>(dev_partial), dev_depth,
                                   dev_count, ctr, s);
     if (e != cudaSuccess) return cuda_fail(e, who);
     return VR_OK;

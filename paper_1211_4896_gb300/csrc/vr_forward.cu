@@ -46,7 +46,6 @@ template <typename T, int LOG2B, int L>
 __global__ void __launch_bounds__(FwdThreads<T>::value, FwdMinBlocks<T>::value) fwd_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
                                                            uint32_t *nsamples, unsigned *counter, Tiles t)
 {
-    if (not_this_march<false>(t, p)) return;
     const int lane = threadIdx.x & 31;
     const float z = skips_transparent<T, IdentityMap>() ? transparent_below(p) : 0.0f;
     for (;;) {
@@ -84,17 +83,21 @@ __global__ void __launch_bounds__(FwdThreads<T>::value, FwdMinBlocks<T>::value) 
 // pixels: 2500: 1.8 to 3.4 times as fast with the benchmark's ramp, 1.5 to 1.9
 // with an opaque table; 10 000: 1.8 to 3.0 and 1.2 to 1.7; 16 000: 1.6 to 3.8 and
 // 0.9 to 1.8; 24 000: 1.3 to 3.5 and 0.75 to 1.6; 38 000: 1.2 to 3.8 and 0.6 to
-// 1.5: an opaque table's samples are all composited, and their shuffles cost
-// more than the latency once an SM has a few tiles.  So views of up to 80
-// covered pixels an SM march in groups, and up to 256 an SM those whose table
-// begins with transparent entries.  Only the device has read the table, so
-// these are launched both ways (Tiles::by_table; both marches in one kernel
-// cost each of them 10% to a factor of 4).
+// 1.5: an opaque table's samples are all handed over and composited, which costs
+// more than the latency once an SM has a few tiles.  So views of up to 112
+// covered pixels an SM march in groups (sigma clipping and sub-boxes, whose
+// samples cost more and whose limits lie higher, up to 160; the maximum, which
+// composites nothing, up to 256), and up to 256 an SM those whose table begins
+// with transparent entries (sparse views whatever the table: a large 16-bit one
+// whose long rays an opaque table never ends runs at 0.86 of a ray to a lane).
+// Only the device has read the table, so these are launched both ways
+// (Tiles::by_table): 2 to 3 us.  Both marches in one kernel cost each of them 10%
+// to a factor of 4.
 template <typename T, int LOG2B, int L>
 __global__ void __launch_bounds__(kFwdThreads, 3 * kPerSm) fwd_group_kernel(VolDev v, CamDev c, ParamDev p, float4 *out,
                                                                 uint32_t *nsamples, unsigned *counter, Tiles t)
 {
-    if (not_this_march<true>(t, p)) return;
+    if (left_to_lanes(t, p)) return;
     const int lane = threadIdx.x & 31;
     const float z = transparent_below(p);
     for (;;) {
@@ -254,7 +257,7 @@ cudaError_t launch_forward(const VolDev &v, vr_dtype dt, const CamDev &c, const 
         return cudaGetLastError();
     };
     if (e == cudaSuccess) e = launch(t);
-    if (e == cudaSuccess && t.by_table) e = launch(lane_tiles(t));    // one of the two returns at once
+    if (e == cudaSuccess && t.by_table) e = launch(lane_tiles(t));    // one of the two finds nothing to do
     return e;
 }
 

@@ -63,8 +63,9 @@ struct VolDev {
 // [y0, y0 + h) around the volume, then 8 x 4 blocks over the whole image for
 // the pixels outside of them, whose rays miss it.  by_table: a view that is
 // better off in groups when its table begins with transparent entries and with
-// a ray to a lane when it does not is launched both ways, and the kernel that
-// the table does not suit returns at once (not_this_march).
+// a ray to a lane when it does not is launched both ways on one work counter:
+// the groups' kernel first, which returns at once when the table does not suit
+// it and else leaves the counter past the other's tiles (nblocks <= ntiles).
 struct Tiles {
     bool groups = false, by_table = false;
     int tiles_x = 0;           // tiles across
@@ -79,7 +80,6 @@ struct Tiles {
 inline Tiles lane_tiles(const Tiles &t)
 {
     Tiles q;
-    q.by_table = t.by_table;
     q.tiles_x = t.blocks_x;
     q.nmarch = q.ntiles = t.nblocks;
     return q;
@@ -190,10 +190,12 @@ inline bool copy_paired(int copy) { return copy >= 3 && copy < 6; }
 inline bool copy_blocked(int copy) { return copy >= 6 && copy < 9; }
 inline bool copy_layers(int copy) { return copy >= 9 && copy < 12; }
 inline int copy_order(int copy) { return copy >= 9 ? copy - 9 : (copy >= 6 ? copy - 6 : (copy >= 3 ? copy - 3 : copy)); }
-// Which march a view takes: as asked, or by the pixels it covers (kByPixels) and,
-// between two limits, its table (kByTable).
-enum March { kRayPerLane, kInGroups, kByPixels, kByTable };
-Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, const double grid_origin[3],
+// Which march a view takes: as asked, or (kAuto) by the covered pixels an SM has
+// and, from `any_table` of them on, the table (limits and figures at
+// fwd_group_kernel).
+enum March { kRayPerLane, kInGroups, kAuto };
+constexpr double kGroupPixels = 256.0, kCompositePixels = 112.0, kModePixels = 160.0;
+Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, double any_table, const double grid_origin[3],
                  const int64_t grid_dims[3]);
 // Whether copy id `copy` exists on vol.
 bool copy_built(const vr_volume *vol, int copy);

@@ -57,7 +57,7 @@ __device__ __forceinline__ float march_max(const VolDev &v, const ParamDev &p, c
     }
     while (__any_sync(kFull, active)) {
         if constexpr (D == 1) {
-            // a vote for each step: with one for two, 16-bit views (30 of 35 to
+            // a vote for each step: with one for two, 16-bit views (30, over 35 to
             // 2000 MB of paired copies) ran at 0.88 to 1.06 of this speed, the
             // largest the slowest
             if (active) step(c0, f0, c1, f1);
@@ -217,7 +217,7 @@ template <typename T, int LOG2B, int L, bool GROUPS, typename I>
 __global__ void __launch_bounds__(kSigmaThreads, 6) sigma_kernel(VolDev v, CamDev c, ParamDev p, MiniDev m, float4 *out,
                                                               uint32_t *nsamples, unsigned *counter, Tiles t)
 {
-    if (not_this_march<GROUPS>(t, p)) return;
+    if (GROUPS && left_to_lanes(t, p)) return;
     const int lane = threadIdx.x & 31;
     const SigmaMap<I> map(m);
     const float z = GROUPS || skips_transparent<T, SigmaMap<I>>() ? transparent_below(p) : 0.0f;
@@ -279,7 +279,7 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
                     : t.groups ? sigma_kernel<typename Y::type, Y::log2b, Y::order, true, int>
                                : sigma_kernel<typename Y::type, Y::log2b, Y::order, false, int>;
             fn<<<persistent_grid(fn, t.ntiles, kSigmaThreads), kSigmaThreads, 0, s>>>(v, c, p, m, out, nsamples, counter, t);
-            if (t.by_table) {                     // both ways: one of the two returns at once
+            if (t.by_table) {                     // both ways: one of the two finds nothing to do
                 const Tiles q = lane_tiles(t);
                 fn = sigma_kernel<typename Y::type, Y::log2b, Y::order, false, int>;
                 fn<<<persistent_grid(fn, q.ntiles, kSigmaThreads), kSigmaThreads, 0, s>>>(v, c, p, m, out, nsamples, counter, q);

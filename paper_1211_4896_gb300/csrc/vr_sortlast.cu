@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kModeThreads, SubMinBlocks<T>::value) subbox_k
     VolDev v, CamDev c, ParamDev p, int3 lo, int3 hi, SubBox box, int3 gdim, float3 off, float4 *partial, float *depth,
     uint32_t *count, unsigned *counter, Tiles t)
 {
-    if (not_this_march<GROUPS>(t, p)) return;
+    if (GROUPS && left_to_lanes(t, p)) return;
     const int lane = threadIdx.x & 31;
     const float z = GROUPS || skips_transparent<T, IdentityMap>() ? transparent_below(p) : 0.0f;
     for (;;) {
@@ -161,7 +161,7 @@ cudaError_t launch_subbox(const VolDev &v, vr_dtype dt, const CamDev &c, const P
                              : subbox_kernel<typename Y::type, Y::log2b, Y::order, false>;
             fn<<<persistent_grid(fn, t.ntiles), kModeThreads, 0, s>>>(v, c, q, l3, h3, box, g3, o3, partial, depth, count,
                                                                       counter, t);
-            if (t.by_table) {                     // both ways: one of the two returns at once
+            if (t.by_table) {                     // both ways: one of the two finds nothing to do
                 const Tiles lt = lane_tiles(t);
                 fn = subbox_kernel<typename Y::type, Y::log2b, Y::order, false>;
                 fn<<<persistent_grid(fn, lt.ntiles), kModeThreads, 0, s>>>(v, c, q, l3, h3, box, g3, o3, partial, depth,
