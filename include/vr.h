@@ -333,9 +333,10 @@ typedef struct {
 
 typedef struct {
     int use_graph;            /* 1: build a CUDA graph of the call on first use (counter reset, then
-                                 one kernel node per brick layout, the layouts running concurrently)
-                                 and replay it while the job list is unchanged (same pointers and
-                                 parameters); 0: launch the layouts one after another */
+                                 one kernel node per brick layout, the layouts running concurrently;
+                                 or one single-view node per job, see vr_render_batched) and replay
+                                 it while the job list is unchanged (same pointers and parameters);
+                                 0: launch the layouts one after another */
     int tile_w, tile_h;       /* ray tile of one warp: tile_w * tile_h == 32; 0 = 8 x 4 */
     int ctas_per_sm;          /* persistent CTAs per SM; 0 = occupancy limit */
     int warps_per_tile;       /* 1, 2 or 4 warps of a CTA take one tile of tile_w x (tile_h x
@@ -348,11 +349,15 @@ typedef struct {
  * the named fields of its jobs (never the structs' padding): the first call
  * with a new list on a stream uploads its descriptors (synchronising
  * cuda_stream); with use_graph the first call also builds the graph.  A list
- * owns one work counter, so the same list on two streams gets two plans.
- * Past 64 cached lists the cache is emptied after a device synchronisation.  Within a layout the jobs
- * with the most work (pixels x samples along the box diagonal) are handed out
- * first.  Later calls with the same list only launch.  Errors: INVALID_ARG,
- * UNSUPPORTED, OOM, CUDA. */
+ * owns its work counters, so the same list on two streams gets two plans.
+ * Past 64 cached lists the cache is emptied after a device synchronisation.
+ * Within a layout the jobs with the most work (pixels x samples along the box
+ * diagonal) are handed out first.  With use_graph and default options, a list
+ * of at most 256 jobs whose float views have 8192 tiles of 8 x 4 pixels on
+ * average, or of which half are sparse (see vr_view_layout), holds one
+ * single-view kernel and counter per job instead, over all layouts in the order
+ * of their work; the images are the same bits.  Later calls with the same list
+ * only launch.  Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
 vr_status vr_render_batched(const vr_job *jobs, int n, const vr_batch_opts *opts, void *cuda_stream);
 
 /* Times candidate tile shapes, CTA counts and warps per tile for this job
@@ -375,7 +380,8 @@ vr_status vr_autotune_batched(const vr_job *jobs, int n, vr_batch_opts *best, vo
  * every GPU that loads the library until the process exits), uploads the
  * descriptors with cudaMemcpyAsync and zeroes the work counters with
  * cudaMemsetAsync on cuda_stream.  The caller still passes the volumes and the
- * outputs.  Jobs are rendered exactly as by vr_render_batched (same kernels);
+ * outputs.  Images and sample counts are the same bits as vr_render_batched's
+ * (whose graphs may hold other kernels for the same jobs);
  * tile_w x tile_h is the warp's ray tile (0, 0 = 8 x 4).  It never builds a
  * brick copy (see vr_volume_create): a view reads such a copy only when an
  * earlier call built it.
