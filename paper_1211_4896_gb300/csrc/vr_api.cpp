@@ -414,26 +414,53 @@ bool sparse_view(const vr_volume *vol, const vr_camera *cam)
     return ray_pitch_voxels(vol, cam, r) >= sparse_min_pitch();
 }
 
-// Whether a view is marched with several lanes to a ray: its rays share no
-// sectors, or it covers few pixels (kGroupPixels an SM; from any_table an SM on
-// only with a table that suits: by_table).
-// VR_GROUPS=0 or 1 (read at each call) has every view marched with a ray to a
-// lane, or in groups: the same images, so that tests reach both marches at any
-// size.  rect: NULL when any pixel may see the volume.
+// Pixels of the image inside the rectangle around the volume (NULL: any pixel
+// may see it).
+static double covered_pixels(const vr_camera *cam, const CornerRect *rect)
+{
+    if (!rect) return (double)cam->width * cam->height;
+    double n = 1.0;
+    for (int a = 0; a < 2; ++a)
+        n *= std::fmax(std::fmin(rect->hi[a], a ? cam->height : cam->width) - std::fmax(rect->lo[a], 0.0), 0.0);
+    return n;
+}
+
+// Whether a sparse view marches in groups: it covers few pixels, or its rays
+// advance along the rows of the layout it reads (the axis nearest to the image's
+// horizontal, see preferred_copy), so that a ray's consecutive samples lie in
+// one sector.  Rays across the rows need a sector a sample either way.  Views of
+// 2048 x 2048 x 1024 and 4096 x 4096 x 1024 cubes in 64^3 bricks, float and
+// float16, against a ray to a lane, with the benchmark's ramp and an opaque
+// table: 45 degrees to the rows, 200 to 3200 covered pixels an SM: 1.15 to 1.56
+// and 0.96 to 1.35 times as fast; across them, 230: 1.04 to 2.0 and 1.0 to 1.08;
+// 950: 1.05 to 1.15 and 0.80 to 1.02; 1650 to 3700: 0.66 to 0.99 and 0.44 to 0.87.
+static bool sparse_in_groups(const vr_volume *vol, const vr_camera *cam, double covered)
+{
+    if (!sparse_view(vol, cam)) return false;
+    if (covered < kSparsePixels * (double)sm_count()) return true;
+    double r[3], f2 = 0.0, along = 0.0, best = -1.0;
+    cross3(cam->forward, cam->up, r);
+    for (int a = 0; a < 3; ++a) {
+        const double c = std::fabs(r[a]) / vol->spacing[a], f = cam->forward[a] / vol->spacing[a];
+        f2 += f * f;
+        if (c > best * (1.0 + 1e-9)) best = c, along = f;
+    }
+    return along * along >= 0.0625 * f2;           // 14 degrees out of the plane across the rows
+}
+
+// Whether a view is marched with several lanes to a ray: it is sparse and gains
+// by it, or it covers few pixels (kGroupPixels an SM; from any_table an SM on
+// only with a table that suits: by_table).  VR_GROUPS=0 or 1 (read at each call)
+// has every view marched with a ray to a lane, or in groups: the same images, so
+// that tests reach both marches at any size.
 static bool march_in_groups(const vr_volume *vol, const vr_camera *cam, const CornerRect *rect, double any_table,
                             bool &by_table)
 {
     by_table = false;
     const char *e = std::getenv("VR_GROUPS");
     if (e && (e[0] == '0' || e[0] == '1')) return e[0] == '1';
-    double covered = (double)cam->width * cam->height;
-    if (rect) {
-        covered = 1.0;
-        for (int a = 0; a < 2; ++a)
-            covered *= std::fmax(std::fmin(rect->hi[a], a ? cam->height : cam->width) - std::fmax(rect->lo[a], 0.0), 0.0);
-    }
-    const double sms = (double)sm_count();
-    if (covered < any_table * sms || sparse_view(vol, cam)) return true;
+    const double covered = covered_pixels(cam, rect), sms = (double)sm_count();
+    if (covered < any_table * sms || sparse_in_groups(vol, cam, covered)) return true;
     return by_table = covered < kGroupPixels * sms;
 }
 
@@ -454,6 +481,7 @@ Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, double
     Tiles t;
     t.groups = march == kInGroups;
     if (march == kAuto) t.groups = march_in_groups(vol, cam, seen ? &q : nullptr, any_table, t.by_table);
+    if (march == kSparse) t.groups = sparse_in_groups(vol, cam, covered_pixels(cam, seen ? &q : nullptr));
     if (!t.groups) {
         t.tiles_x = (W + 7) / 8;
         t.nmarch = t.ntiles = (unsigned)t.tiles_x * (unsigned)((H + 3) / 4);

@@ -480,7 +480,7 @@ extern "C" vr_status vr_render_batched(const vr_job *jobs, int n, const vr_batch
             for (int q : by_cost) {
                 plan->nodes.push_back(hj[q]);
                 const vr_job &J = jobs[order[q]];
-                plan->tiles.push_back(view_tiles(J.vol, &J.cam, sparse_view(J.vol, &J.cam) ? kInGroups : kRayPerLane, 0.0, J.vol->origin,
+                plan->tiles.push_back(view_tiles(J.vol, &J.cam, hj[q].v.paired == 2 ? kInGroups : kSparse, 0.0, J.vol->origin,
                                                  J.vol->dims));
             }
         }

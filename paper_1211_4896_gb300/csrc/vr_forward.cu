@@ -64,8 +64,9 @@ __global__ void __launch_bounds__(FwdThreads<T>::value, FwdMinBlocks<T>::value) 
 
 // Eight lanes to a ray (march_group, kGroup), for two kinds of views:
 //
-// Sparse views (rays three or more voxels apart at the volume centre).  Neighbouring rays share no sectors there, and
-// with a ray to each lane the lines it fetched were evicted before its next
+// Sparse views (rays three or more voxels apart at the volume centre) that cover
+// few pixels or look along the layout's rows (sparse_in_groups has the limits).
+// Neighbouring rays share no sectors there, and with a ray to each lane the lines it fetched were evicted before its next
 // samples came to use them: 59 DRAM bytes a sample against 17 compulsory, the
 // march waiting on memory 12 of 13 issue slots.  Eight consecutive samples of
 // a ray in one warp instruction use a line at once, and an eighth of the rays
@@ -88,8 +89,7 @@ __global__ void __launch_bounds__(FwdThreads<T>::value, FwdMinBlocks<T>::value) 
 // covered pixels an SM march in groups (sigma clipping and sub-boxes, whose
 // samples cost more and whose limits lie higher, up to 160; the maximum, which
 // composites nothing, up to 256), and up to 256 an SM those whose table begins
-// with transparent entries (sparse views whatever the table: a large 16-bit one
-// whose long rays an opaque table never ends runs at 0.86 of a ray to a lane).
+// with transparent entries (sparse views: sparse_in_groups).
 // Only the device has read the table, so these are launched both ways
 // (Tiles::by_table): 2 to 3 us.  Both marches in one kernel cost each of them 10%
 // to a factor of 4.

@@ -190,11 +190,12 @@ inline bool copy_paired(int copy) { return copy >= 3 && copy < 6; }
 inline bool copy_blocked(int copy) { return copy >= 6 && copy < 9; }
 inline bool copy_layers(int copy) { return copy >= 9 && copy < 12; }
 inline int copy_order(int copy) { return copy >= 9 ? copy - 9 : (copy >= 6 ? copy - 6 : (copy >= 3 ? copy - 3 : copy)); }
-// Which march a view takes: as asked, or (kAuto) by the covered pixels an SM has
+// Which march a view takes: as asked, in groups if it is sparse and gains by it
+// (kSparse, sparse_in_groups), or (kAuto) also by the covered pixels an SM has
 // and, from `any_table` of them on, the table (limits and figures at
 // fwd_group_kernel).
-enum March { kRayPerLane, kInGroups, kAuto };
-constexpr double kGroupPixels = 256.0, kCompositePixels = 112.0, kModePixels = 160.0;
+enum March { kRayPerLane, kInGroups, kSparse, kAuto };
+constexpr double kGroupPixels = 256.0, kCompositePixels = 112.0, kModePixels = 160.0, kSparsePixels = 1000.0;
 Tiles view_tiles(const vr_volume *vol, const vr_camera *cam, March march, double any_table, const double grid_origin[3],
                  const int64_t grid_dims[3]);
 // Whether copy id `copy` exists on vol.

@@ -295,9 +295,9 @@ cudaError_t launch_sigma(const VolDev &v, vr_dtype dt, const CamDev &c, const Pa
 //
 // FP64 adds and fused multiply-adds run at two lanes per clock and SM here:
 // two passes of them take 5.1 ms for a 768^3 float cube in regions of 32^3,
-// where reading its bricks takes 0.33 ms; this takes 0.96 ms (1.55 with a NaN
-// in every region, 1.86 where every region takes the second pass below), bound
-// by FP32 instructions.  So a region is read once, and its sums of
+// where reading its bricks takes 0.33 ms; this takes 0.94 ms (1.8 with a NaN in
+// every region, 2.1 where every region takes the second pass below), bound by
+// FP32 instructions.  So a region is read once, and its sums of
 // d = a - shift and of d^2 (shift: the region's first voxel) are kept as
 // unevaluated sums of two floats, with the rounding errors of every
 // subtraction, product and addition carried along (Knuth's two-sum and the
